@@ -2,18 +2,20 @@
 //
 // On GB300 the FP64 pipe retires 2 lanes per SM per clock while the integer
 // and FP32 pipes retire 64-128; the stage kernel is bound by FP64 issue.  So:
-//  * reciprocal and (reciprocal) square root start from the hardware's
-//    documented approximations (PTX rcp.approx.ftz.f64, rsqrt.approx.ftz.f64)
-//    and are refined by ONE third-order Newton-Raphson / series step (the
-//    classical iteration for 1/x and 1/sqrt(x), see e.g. Muller et al.,
-//    Handbook of Floating-Point Arithmetic, ch. 5): with the residual
-//    e = 1 - x y0 (resp. 1 - x y0^2),
-//        1/x       = y0 (1 + e + e^2 + ...)
+//  * reciprocal and square root are computed on the integer pipes
+//    (gbh_intmath.cuh), within 0.52 and 0.56 ulp.  They took 3 and 5 FP64
+//    instructions of 64 issue cycles each; 29 of the 80 a face needs.  3-D step
+//    of 256^3: 20.88 -> 16.71 ms, of 128^3: 3.105 -> 2.495 ms, 96-problem 2-D
+//    ensemble 8.52 -> 6.88 ms.
+//  * the reciprocal square root (the adjoint's) starts from the hardware's
+//    documented approximation (PTX rsqrt.approx.ftz.f64) and is refined by ONE
+//    third-order series step (the classical iteration, see e.g. Muller et al.,
+//    Handbook of Floating-Point Arithmetic, ch. 5): with e = 1 - x y0^2,
 //        1/sqrt(x) = y0 (1 + e/2 + 3 e^2/8 + ...),
 //    truncated after the quadratic term, so the relative error of the seed
-//    is cubed; the results are within a few ulp of the correctly rounded
-//    ones (not bit-identical to IEEE division / sqrt).  Valid for positive,
-//    normal, finite inputs -- what the scheme feeds them.
+//    is cubed; within a few ulp of the correctly rounded result.
+//    All three take positive (the reciprocal: also negative), normal, finite
+//    inputs -- what the scheme feeds them.
 //  * comparisons, min / max and sign tests of doubles are done on the bit
 //    patterns with 64-bit integer operations (ALU pipe), which give the same
 //    decisions as the IEEE comparisons for non-NaN values.
@@ -36,6 +38,7 @@
 #include <stdint.h>
 
 #include "gbh_internal.h"
+#include "gbh_intmath.cuh"
 
 namespace gbh {
 
@@ -93,25 +96,25 @@ __device__ __forceinline__ double quarter_any(double x) {
   return bitsd(m2 >= (6ULL << 52) ? dbits(x) - (2LL << 52) : (long long)(sign_bit(x) | (m2 >> 3)));
 }
 
-__device__ __forceinline__ double rcp_approx(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-
 __device__ __forceinline__ double rsqrt_approx(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   return y;
 }
 
-// 1/x: 3 FP64 operations after the seed.
-__device__ __forceinline__ double rcp_nr(double x, const Rk& k) {
-  const double y = rcp_approx(x);
-  const double e = fma(-x, y, k.one);
-  const double t = fma(e, e, e);
-  return fma(y, t, y);
+// The unpacked magnitude of x, and x from a bit pattern held as two words.
+__device__ __forceinline__ Wide wide_of(double x) {
+  return wide_unpack((uint32_t)((unsigned long long)dbits(x) >> 32), (uint32_t)dbits(x));
 }
+
+// 1/x on the integer pipes (gbh_intmath.cuh), within 0.52 ulp: no FP64
+// operation (3 before).  NaN for zeros, subnormals, infinities, NaN and |x| >= 2^1022.
+__device__ __forceinline__ double rcp_nr(double x) {
+  const Wide a = wide_of(x);
+  const long long r = (long long)(wide_pack(wide_rcp(a)) | sign_bit(x));
+  return bitsd((unsigned)(a.e - 1) < 2044u ? r : 0x7ff8000000000000LL);
+}
+__device__ __forceinline__ double rcp_nr(double x, const Rk&) { return rcp_nr(x); }
 
 // The series term e/2 + 3e^2/8 of the square-root refinements, as h + (3/2) h^2
 // with h = e/2 (exponent decrement on the integer pipe): 2 FP64 operations.
@@ -128,17 +131,16 @@ __device__ __forceinline__ double rsqrt_nr(double x, const Rk& k) {
   return fma(y, rsqrt_corr(e, k), y);
 }
 
-// sqrt(x) = x / sqrt(x), refined the same way: 5 FP64 operations after the seed.
-__device__ __forceinline__ double sqrt_nr(double x, const Rk& k) {
-  const double y = rsqrt_approx(x);
-  const double t = mul(x, y, k);
-  const double e = fma(-t, y, k.one);
-  return fma(t, rsqrt_corr(e, k), t);
+// sqrt(x) on the integer pipes (gbh_intmath.cuh), within 0.56 ulp: no FP64
+// operation (5 before).  NaN for zeros, subnormals, negative values, infinities and NaN.
+__device__ __forceinline__ double sqrt_nr(double x) {
+  const Wide a = wide_of(x);
+  const unsigned field = (unsigned)((unsigned long long)dbits(x) >> 52);   // sign and exponent
+  return bitsd(field - 1u < 2046u ? (long long)wide_pack(wide_sqrt(a)) : 0x7ff8000000000000LL);
 }
+__device__ __forceinline__ double sqrt_nr(double x, const Rk&) { return sqrt_nr(x); }
 
-__device__ __forceinline__ double rcp_nr(double x) { return rcp_nr(x, plain_rk()); }
 __device__ __forceinline__ double rsqrt_nr(double x) { return rsqrt_nr(x, plain_rk()); }
-__device__ __forceinline__ double sqrt_nr(double x) { return sqrt_nr(x, plain_rk()); }
 
 // ---- integer-domain comparisons -------------------------------------------
 
