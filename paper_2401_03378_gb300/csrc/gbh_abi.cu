@@ -524,6 +524,13 @@ void layout_from_params(const gbh_params* p, Layout* L, Eos* e) {
   e->k.one = 1.0;
   e->k.nz = -0.0;
   e->opaque = 0;
+  auto unpacked = [](double x) {
+    uint64_t u;
+    memcpy(&u, &x, sizeof u);
+    return wide_unpack((uint32_t)(u >> 32), (uint32_t)u);
+  };
+  e->wgamma = unpacked(e->gamma);
+  e->whgm1 = unpacked(e->hgm1);
 }
 
 void face_table_from_params(const gbh_params* p, long long b, int face[6], double inv_dx[3]) {

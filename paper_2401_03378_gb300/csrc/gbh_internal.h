@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/gbhydro.h"
+#include "gbh_intmath.cuh"
 
 namespace gbh {
 
@@ -33,6 +34,7 @@ struct Eos {
   double gamma, gm1, inv_gm1, g_gm1, small_rho, small_p;  // g_gm1 = gamma / (gamma - 1)
   double hgm1;                                            // (gamma - 1) / 2
   Rk k;                                                   // {1, -0}
+  Wide wgamma, whgm1;                                     // gamma and (gamma - 1) / 2 unpacked (gbh_intmath.cuh)
   long long opaque;                                       // 0 (see reg_eos)
 };
 
