@@ -121,8 +121,38 @@ __device__ __forceinline__ double block_max(double v, double* s_warp) {
 // Wide -> double, for a result in the normal range.
 __device__ __forceinline__ double wide_double(const Wide& a) { return bitsd((long long)wide_pack(a)); }
 
-// Infinity or NaN.
-__device__ __forceinline__ bool not_finite(double x) { return (unsigned)((mag_key(x) >> 32)) >= 0xffe00000u; }
+__device__ __forceinline__ uint32_t hi_word(double x) { return (uint32_t)((unsigned long long)dbits(x) >> 32); }
+
+// The unpacked magnitude of x, with zeros (and subnormals) as numbers so small
+// that no product of the scheme brings them back into the range of a double.
+__device__ __forceinline__ Wide wide_of0(double x) {
+  Wide a = wide_of(x);
+  a.e = a.e == 0 ? -8192 : a.e;
+  return a;
+}
+
+// Wide -> double with the sign bit (and, for a NaN, the exponent bits) of `top`
+// OR-ed in: below the normal range a zero, above it a NaN.
+__device__ __forceinline__ double wide_signed(const Wide& a, uint32_t top) {
+  const uint64_t m = wide_pack(a);
+  uint32_t h = imath::hi32(m), l = imath::lo32(m);
+  const bool in = (unsigned)(a.e - 1) < 2045u;
+  const uint32_t out = a.e < 1 ? 0u : 0x7ff80000u;
+  h = (in ? h : out) | top;
+  l = in ? l : 0u;
+  return bitsd((long long)imath::pair(h, l));
+}
+
+// See hllc_flux.
+__device__ __forceinline__ uint32_t non_finite_mask(const double WL[5], const double WR[5]) {
+  float z = 0.0f;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    z = fmaf(__uint_as_float(hi_word(WL[v])), 0.0f, z);
+    z = fmaf(__uint_as_float(hi_word(WR[v])), 0.0f, z);
+  }
+  return __float_as_uint(z);
+}
 
 // Signal-speed sum of one cell for the CFL rule; W from cons_to_prim and
 // ir = 1 / W[0] (cons_to_prim_ir returns it).
@@ -173,14 +203,19 @@ __device__ __forceinline__ double signal_speed_ir(const double W[5], double ir, 
 // roots' and reciprocals' own (64 issue cycles each, against 1 to 2).  The
 // chain carries 57 bits and rounds only its four results.  80 -> 37 FP64
 // instructions a face with the remaining roots and reciprocals; of that the
-// chain: 256^3 step 16.71 -> 14.07 ms, 96-problem 2-D ensemble 6.88 -> 5.71 ms.  An infinity or NaN
-// in a density, a pressure or a normal velocity reaches the flux through the
-// FP64 part as before (m_K, p_R - p_L, u~); |u_L - u_R|^2 hands it to c~.
+// chain: 256^3 step 16.71 -> 14.07 ms, 96-problem 2-D ensemble 6.88 -> 5.71 ms.
+// The quotients S* and t, whose factors are already unpacked, follow the same
+// way (m_L - m_R is a sum of two negative numbers): 37 -> 31 FP64 instructions.
 __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5], const Eos& e,
                                           double F[5]) {
   const Rk& k = e.k;
   const double rL = WL[0], uL = WL[1], vL = WL[2], wL = WL[3], pL = WL[4];
   const double rR = WR[0], uR = WR[1], vR = WR[2], wR = WR[3], pR = WR[4];
+
+  // +0, or a NaN's bits when any input is not finite (FP32 arithmetic on the
+  // high words, whose exponent field is all ones for an infinity, a NaN or a
+  // magnitude from 2^1017): OR-ed into S* and t, from where it reaches every flux
+  const uint32_t bad = non_finite_mask(WL, WR);
 
   // the wave speeds' positive part, on the integer pipes
   const Wide RL = wide_of(rL), RR = wide_of(rR);
@@ -197,22 +232,32 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
   const double du2 = fma(dw, dw, fma(dv, dv, mul(du, du, k)));
   const Wide ct2 = wide_add(wide_mul(wl, cL2),
                             wide_mul(wr, wide_add(cR2, wide_mul(wide_mul(e.whgm1, wl), wide_of(du2)))));
-  const double ct = not_finite(du2) ? du2 : wide_double(wide_sqrt(ct2));
+  const double ct = wide_double(wide_sqrt(ct2));
 
   const double SL = min_d(sub(uL, cL, k), sub(ut, ct, k));
   const double SR = max_d(add(uR, cR, k), add(ut, ct, k));
-  const double dL = sub(SL, uL, k), dR = sub(SR, uR, k);
-  const double mL = mul(rL, dL, k), mR = mul(rR, dR, k);
-  const double Ss = mul(fma(-mR, uR, fma(mL, uL, sub(pR, pL, k))), rcp_nr(sub(mL, mR, k), k), k);
+  const double dL = sub(SL, uL, k), dR = sub(SR, uR, k);   // <= 0 and >= 0
+  const Wide DL = wide_of0(dL), DR = wide_of0(dR);
+  const Wide ML = wide_mul(RL, DL), MR = wide_mul(RR, DR); // |m_L|, |m_R|
+  const double mL = wide_signed(ML, 0x80000000u), mR = wide_signed(MR, 0u);
+  // S* = num / (m_L - m_R) = -num / (|m_L| + |m_R|)
+  const double num = fma(-mR, uR, fma(mL, uL, sub(pR, pL, k)));
+  const Wide WS = wide_mul(wide_of0(num), wide_rcp(wide_add(ML, MR)));
+  const uint32_t sgn = ~hi_word(num) & 0x80000000u;
+  const double Ss = wide_signed(WS, sgn | bad);
 
   const bool left = ge0(Ss);
   const double rK = sel(left, rL, rR), uK = sel(left, uL, uR), vK = sel(left, vL, vR);
   const double wK = sel(left, wL, wR), pK = sel(left, pL, pR);
-  const double SK = sel(left, SL, SR), mK = sel(left, mL, mR), dK = sel(left, dL, dR);
+  const double SK = sel(left, SL, SR), mK = sel(left, mL, mR);
   const bool fan = left ? lt0(SL) : gt0(SR);
 
   // t = u_K + g; S_K - S* != 0 inside the fan, and t = u_K (g = 0) outside it
-  const double t = sel(fan, mul(Ss, mul(dK, rcp_nr(sub(SK, Ss, k), k), k), k), uK);
+  const double SKs = sub(SK, Ss, k);
+  const Wide DK = left ? DL : DR;
+  const Wide T = wide_mul(wide_mul(WS, DK), wide_rcp(wide_of(SKs)));
+  const uint32_t tsgn = (sgn ^ hi_word(SKs) ^ (left ? 0x80000000u : 0u)) & 0x80000000u;
+  const double t = sel(fan, wide_signed(T, tsgn | bad), uK);
   const double g = sub(t, uK, k);
   // E + p of the chosen side (rho >= small_rho, a normal number)
   const double hK = fma(half_pos(rK), fma(wK, wK, fma(vK, vK, mul(uK, uK, k))), mul(e.g_gm1, pK, k));
