@@ -531,6 +531,7 @@ void layout_from_params(const gbh_params* p, Layout* L, Eos* e) {
   };
   e->wgamma = unpacked(e->gamma);
   e->whgm1 = unpacked(e->hgm1);
+  e->wg_gm1 = unpacked(e->g_gm1);
 }
 
 void face_table_from_params(const gbh_params* p, long long b, int face[6], double inv_dx[3]) {
