@@ -262,6 +262,12 @@ def make_problem(nb: int):
     return lat, wl.sedov(lat)
 
 
+def prepass_runs(h):
+    """Whether the stages of a context with default settings launch the face pre-pass
+    (by default only for blocks narrower than 16 cells)."""
+    return h.face_prepass() and h.n[0] < 16
+
+
 def fp64_probe_tflops(gb, torch, form=1):
     """FP64 flop/s of the probe's fused multiply-add chains: form 1 with all
     operands in registers (the fastest form), form 0 with constant operands."""
@@ -438,7 +444,7 @@ def run_gpu(args):
     roof = {
         "kernel": ("gbh face_flux_kernel<16,3D> + stage_kernel<16,3D> per stage, timed together (both SSP-RK2 "
                    "stages: each block face solved once in the pre-pass, fused halo gather, dt epilogue)"
-                   if h.face_prepass() else
+                   if prepass_runs(h) else
                    "gbh stage_kernel<16,3D> (both SSP-RK2 stages, fused halo gather, dt epilogue)"),
         "bound": "alu",
         "achieved": achieved / 1e12,
@@ -473,7 +479,7 @@ def run_gpu(args):
         "data": "synthetic (seeded Sedov initial condition)",
         "config": bench_config(lat),
         "parallelism": f"replicas x{world}",
-        "gpu_launches": (5 if h.face_prepass() else 3) * args.steps,
+        "gpu_launches": (5 if prepass_runs(h) else 3) * args.steps,
         "autotune": tuning,
         "clocks": clocks,
         "repeats": repeats,
@@ -546,7 +552,7 @@ def run_variants(args, gb, torch, barrier, ms_headline):
         stage_ms, _ = h.stage_kernel_time()
         h.set_kernel_timing(False)
         nbad = h.check_state(U)
-        pre = h.face_prepass() and not tele      # the face pre-pass runs before halo-gathering stages
+        pre = prepass_runs(h) and not tele      # the face pre-pass runs before halo-gathering stages
         h.close()
         del U
         torch.cuda.empty_cache()
@@ -600,7 +606,7 @@ def run_two_level(args, gb, torch, barrier):
     barrier()
     tsecs = e0.elapsed_time(e1) / 1e3
     tbad = h.check_state(U)
-    pre = 2 if h.face_prepass() else 0     # the face pre-pass of the two all-levels stages
+    pre = 2 if prepass_runs(h) else 0     # the face pre-pass of the two all-levels stages
     h.close()
     del U
     torch.cuda.empty_cache()
@@ -718,7 +724,7 @@ def run_two_level_ensemble(args, gb, torch, barrier):
     h.compute_dt(U, dt)
     batched = timed(lambda: h.advance_graph(U, n, dt))
     nbad = h.check_state(U)
-    pre = 2 if h.face_prepass() else 0     # the face pre-pass of the two stages
+    pre = 2 if prepass_runs(h) else 0     # the face pre-pass of the two stages
     h.close()
     del U
     torch.cuda.empty_cache()

@@ -143,7 +143,8 @@ int gbh_create_refined_batched(const gbh_params *params, const gbh_refinement *r
 
 /* Work decomposition of the stage kernel (how the concurrent-data pattern of
  * Sec. 3.2 maps blocks onto CTAs; not a choice the paper makes): kchunk = z planes per work item
- * (3-D; 0 or nzb = the whole block) and items_per_cta = consecutive work
+ * (3-D; 0 or nzb = the whole block; a new context picks it per launch from
+ * the number of blocks and SMs) and items_per_cta = consecutive work
  * items one CTA processes (1 = a CTA per item; a grid of about two CTAs per
  * SM makes the kernel persistent).  A third choice is the tile: the plane
  * tile of a work item (the nxb x nyb block plane, widened by the ring in the
@@ -249,7 +250,9 @@ int gbh_get_prim_carry(gbh_ctx *ctx, int *enabled);
  * HLLC arithmetic).  Every gbh_create* allocates its buffer ([nblocks][6]
  * [5][nxb max(nxb, nzb)] doubles) and switches it on for 3-D contexts (off
  * if that allocation fails); 2-D contexts start with it off (enable
- * allocates [nblocks][6][5][nxb] doubles).  enable = 0 switches it off (the
+ * allocates [nblocks][6][5][nxb] doubles).  On by default it runs where it
+ * pays, for blocks narrower than 16 cells in whole-block work items; after a
+ * call with enable != 0 it runs at every width.  enable = 0 switches it off (the
  * buffer stays).  GBH_ERR_NOMEM if enable != 0 and the buffer cannot be
  * allocated.  Drops a captured graph. */
 int gbh_set_face_prepass(gbh_ctx *ctx, int enable);

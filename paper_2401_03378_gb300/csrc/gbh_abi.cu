@@ -41,6 +41,7 @@ struct gbh_ctx {
   // fluxes through every block face, [nblocks][6][5][nx * nx (3-D) or nx]
   double* d_bflux = nullptr;
   bool face_prepass = false;
+  bool prepass_asked = false;       // switched on by the caller: used at every block width
   unsigned long long* d_words = nullptr;  // [0] smax accumulator, [1] floor count, [2] check count
   // host-buffer path (allocated on first use)
   double* d_host_state = nullptr;
@@ -70,7 +71,8 @@ struct gbh_ctx {
   unsigned long long* d_smax = nullptr;  // [nproblems]; points into d_words for a single problem
   unsigned long long* d_smax_own = nullptr;
   // stage-kernel work decomposition (gbh_autotune)
-  int kchunk = 0;                   // z planes per work item (3-D); 0 = the whole block
+  int kchunk = -1;                  // z planes per work item (3-D); 0 = the whole block, -1 = by auto_kchunk
+  int sms = 0;                      // SMs of the device
   int items_per_cta = 1;
   int ysplit[3] = {1, 1, 1};        // row bands of the plane tile for ring widths 0, 2, 4
   // CUDA graph of hydro_advance_graph
@@ -166,6 +168,39 @@ int record_start(gbh_ctx* c, cudaStream_t s, cudaEvent_t* stop) {
   return cuda_err(c, cudaEventRecord(a, s), "cudaEventRecord");
 }
 
+// z planes per work item of a stage over nblk blocks of `span` planes with
+// `threads` threads per CTA, where the caller has set no decomposition.  A CTA
+// marches through its planes one after another, so with few blocks most of the
+// chip idles behind the march (eight 16^3 blocks: 8 of 152 SMs) and with a few
+// more the last wave is nearly empty (512 blocks on 152 SMs: 4 rounds of work
+// where 3.37 would do).  A chunk repeats the slopes and the face at its lower
+// end, about 0.8 of a plane.  The time of a chunking is therefore taken as
+// (k + 0.8) max(10, w m): m items on the busiest SM, w warps per item; a lone CTA
+// of any size takes about as long for a plane as 10 warps' share of a full SM
+// (measured, 16^3 and 8^3 blocks: 18 us a plane alone, 14 us per 8 warps when
+// full).  Against whole blocks, us per step of two stages (in brackets the k
+// chosen here): 8 blocks of 16^3 604 -> 68 (1), 27: 609 -> 143 (1), 125: 641 -> 481
+// (8), 512: 1844 -> 1686 (8), 990: 3251 (16); 105 blocks of 8 x 8 x 12: 408 -> 131
+// (2), 512 of 8^3 360 -> 296 (4), 990: 529 (8); telescoping, 216 blocks of 16^3: 1474
+// -> 1189.  Over the k measured beside it (2, 3, 4, 6, 8 and whole blocks) the choice
+// is the fastest, or within 10% of it.
+int auto_kchunk(int span, long long nblk, int threads, int sms) {
+  const double w = threads > 32 ? threads / 32.0 : 1.0;
+  int best = span;
+  double best_t = 1e300;
+  for (int n = 1; n <= span; ++n) {
+    const int k = (span + n - 1) / n;
+    const long long items = nblk * ((span + k - 1) / k);
+    const double m = (double)((items + sms - 1) / sms);
+    const double t = (k + 0.8) * (w * m > 10.0 ? w * m : 10.0);
+    if (t < 0.98 * best_t) {     // a finer cut has to gain more than the estimate is worth
+      best_t = t;
+      best = k;
+    }
+  }
+  return best;
+}
+
 // One stage launch.  ring > 0: the telescoping form that also updates that
 // many guard cells around the interior, from Uin's own guard cells.
 // range_first >= 0: `list` is the identity list of blocks [range_first,
@@ -193,19 +228,28 @@ int stage_launch(gbh_ctx* c, const double* Uin, const double* Un, double* Uout, 
   A.smax_acc = dt_epilogue ? c->d_smax : nullptr;
   A.floor_count = c->d_words + 1;
   A.problem = c->d_problem;
-  if (ring > 0 && c->lay.ndim == 3) {
-    // a ring-updating stage spans nz + 2*ring planes
+  A.ysplit = (ring == 0 || ring == 2 || ring == 4) ? c->ysplit[ring / 2] : 1;
+  // The face pre-pass by default only below 16 cells per side: a block of 16^3
+  // has few boundary faces for what the extra launch and its buffer cost now
+  // that a face takes 19 FP64 instructions (4096 blocks of 16^3: 12.32 ms a step
+  // with it, 12.17 without; 4096 blocks of 8^3: 1.86 and 2.09).
+  const bool prepass = c->face_prepass && c->d_bflux && ring == 0 && gather && (!list || range_first >= 0) &&
+                       A.ysplit == 1 && (c->prepass_asked || c->lay.nx < 16);
+  if (c->lay.ndim == 3) {
+    // a ring-updating stage spans nz + 2*ring planes; with the pre-pass a work
+    // item is a whole block, and so it is in a range of a pipelined stage (one
+    // wave of whole blocks already)
     const int span = c->lay.nz + 2 * ring;
-    A.kchunk = c->kchunk > 0 ? c->kchunk : span;
+    const int side = c->lay.nx + 2 * ring;
+    const long long nblk = list ? nlist : c->refined ? c->nactive : c->lay.nblocks;
+    int k = c->kchunk;
+    if (k < 0)
+      k = (range_first >= 0 || (prepass && c->prepass_asked)) ? span
+                                                              : auto_kchunk(span, nblk, side * side / A.ysplit, c->sms);
+    A.kchunk = k > 0 ? k : span;
     A.nchunks = (span + A.kchunk - 1) / A.kchunk;
-  } else if (c->lay.ndim == 3 && c->kchunk > 0) {
-    A.kchunk = c->kchunk;
-    A.nchunks = (c->lay.nz + c->kchunk - 1) / c->kchunk;
   }
   A.items_per_cta = c->items_per_cta;
-  A.ysplit = (ring == 0 || ring == 2 || ring == 4) ? c->ysplit[ring / 2] : 1;
-  const bool prepass = c->face_prepass && c->d_bflux && ring == 0 && gather && (!list || range_first >= 0) &&
-                       A.ysplit == 1 && A.nchunks == 1;
   if (c->refined) {
     A.block_list = c->d_active;
     A.nlist = c->nactive;
@@ -220,7 +264,7 @@ int stage_launch(gbh_ctx* c, const double* Uin, const double* Un, double* Uout, 
   cudaEvent_t stop;
   int rc = record_start(c, s, &stop);
   if (rc) return rc;
-  if (prepass) {
+  if (prepass && A.nchunks == 1) {
     // each block face solved once, then read by the stage
     const int lo = list ? range_first : 0, hi = list ? range_first + nlist : -1;
     if ((rc = cuda_err(c, gbh::launch_face_fluxes(A, c->d_bflux, s, lo, hi), "face pre-pass launch"))) return rc;
@@ -631,6 +675,7 @@ static int create_common(const gbh_params* p, gbh_ctx** out) {
   for (long long b = 0; b < p->nblocks; ++b) gbh::face_table_from_params(p, b, &face[6 * b], &inv[3 * b]);
 
   cudaError_t e = cudaGetDevice(&c->device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_nbr, sizeof(int) * nn * (size_t)p->nblocks);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_face, sizeof(int) * face.size());
   if (e == cudaSuccess) e = cudaMalloc(&c->d_inv_dx, sizeof(double) * inv.size());
@@ -1085,10 +1130,11 @@ int gbh_set_face_prepass(gbh_ctx* c, int enable) {
   if (rc) return rc;
   drop_graph(c);
   if (!enable) {
-    c->face_prepass = false;
+    c->face_prepass = c->prepass_asked = false;
     return GBH_OK;
   }
   if (!alloc_face_buffer(c)) return set_err(c, GBH_ERR_NOMEM, "face pre-pass buffer: device allocation failed");
+  c->prepass_asked = true;
   return GBH_OK;
 }
 

@@ -646,17 +646,21 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const StageArgs a, doubl
   }
 }
 
-// CTAs per SM the register budget is sized for: an unsplit interior tile
-// (256 threads at N = 16) two, a band of it four; a ring tile one, a band
-// of it two.
-template <int E, int S>
-constexpr int min_ctas() { return (E == 0 ? 2 : 1) * S; }
+// CTAs per SM the register budget is sized for: 512 threads (128 registers
+// each) of interior or small ring tiles; for blocks of 16 an unsplit ring tile
+// one CTA, a band of it two.  (Blocks of 8 were budgeted for two CTAs of 64
+// threads, which left 4 resident and 8 warps per SM.)
+template <int N, int E, int S>
+constexpr int min_ctas() {
+  constexpr int NT = (stage_threads<N, E, S>() + 31) / 32 * 32;
+  return E > 0 && N == 16 ? S : 512 / NT > 1 ? 512 / NT : 1;
+}
 
 // Work list: items (block, z-chunk, band) in order; each CTA processes
 // `items_per_cta` consecutive items (1 = one CTA per item; a machine-sized
 // grid makes the kernel persistent).  No CTA waits on another.
 template <int N, bool DIM3, int E, int S, bool BF = false>
-__global__ void __launch_bounds__(stage_threads<N, E, S>(), min_ctas<E, S>()) stage_kernel(const StageArgs a) {
+__global__ void __launch_bounds__(stage_threads<N, E, S>(), min_ctas<N, E, S>()) stage_kernel(const StageArgs a) {
   constexpr int NT = stage_threads<N, E, S>();
   extern __shared__ double smem[];
   __shared__ double s_red[E == 0 && NT > 32 ? NT / 32 : 1];
