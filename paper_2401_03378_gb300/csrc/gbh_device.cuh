@@ -24,6 +24,12 @@
 
 namespace gbh {
 
+// The bit pattern of x by its two words (the compiler does not look through
+// the intrinsics, so masked sign bits do not become FP64 operations).
+__device__ __forceinline__ uint64_t word_pair(double x) {
+  return imath::pair((uint32_t)__double2hiint(x), (uint32_t)__double2loint(x));
+}
+
 // calcEos role: conserved (rho, mx, my, mz, E) -> primitive (rho, u, v, w, p),
 // p = (gamma-1) (E - (mx u + my v + mz w)/2).  Floors rho at small_rho and p
 // at small_p; returns 1 when a floor applied.
@@ -64,20 +70,12 @@ __device__ __forceinline__ double mc_half_slope(double qm, double q0, double qp)
 // Half the MC-limited slope from the differences dm = q0 - qm, dp = qp - q0:
 //   sigma/2 = sign(dp) * min(|dm+dp|, 4|dm|, 4|dp|) / 4
 // if dm, dp have the same strict sign, else 0, so the face values are
-// q0 -/+ sigma/2 (register FMAs).  The factors 4 are added to the exponent
-// fields of |dm|, |dp| and the division by 4 taken off the exponent of the
-// minimum, on the integer pipe: exact for normal numbers (a subnormal |dm| or
-// |dp|, or a minimum below 2^-1020, is scaled by shifting the bit pattern,
-// which moves the result by less than 2^-1020).  One FP64 operation (the sum).
-__device__ __forceinline__ double mc_half_slope_d(double dm, double dp, const Rk& k) {
-  const double sum = add(dm, dp, k);
-  const unsigned long long am = mag_key(dm), ap = mag_key(dp), as = mag_key(sum);
-  unsigned long long m = (am < ap ? am : ap) + (4ULL << 52);   // min(4|dm|, 4|dp|): exponent + 2 in key form
-  m = as < m ? as : m;
-  m >>= 1;                                                       // magnitude bits of 2 sigma
-  m = m >= (3ULL << 52) ? m - (2ULL << 52) : m >> 2;            // / 4
-  const bool same = ((dbits(dm) ^ dbits(dp)) >= 0) && am != 0 && ap != 0;
-  return bitsd(same ? (long long)(m | sign_bit(dp)) : 0LL);
+// q0 -/+ sigma/2.  On the integer pipes (gbh_intmath.cuh), the bits of the FP64
+// form: the sum there took 64 cycles of the FP64 pipe, here about 24 more integer
+// instructions (256^3 step 12.05 -> 11.72 ms, 96-problem ensemble 5.29 -> 4.98 ms; the
+// face values' two sums cost more as integer work than they free: 13.05 ms).
+__device__ __forceinline__ double mc_half_slope_d(double dm, double dp, const Rk&) {
+  return bitsd((long long)half_slope(word_pair(dm), word_pair(dp)));
 }
 
 // x / 2 for a positive normal x >= 2^-1021 (one off the exponent field)

@@ -213,4 +213,31 @@ GBH_HD Wide wide_sqrt(const Wide& a) {
   return r;
 }
 
+// sign(p) min(|m + p| / 4, |m|, |p|) where the doubles with bit patterns m and p
+// have the same strict sign, else +0: half the MC-limited slope of the
+// differences m and p, |m + p| / 4 rounded once to nearest even (as the FP64 sum
+// would be).  With a <= b the magnitudes, (a + b) / 4 < a needs b < 3 a, so the
+// exponents differ by at most 2 there and the 53-bit mantissas add exactly in 64
+// bits.  For a below 2^-1021 the result is a itself.
+GBH_HD uint64_t half_slope(uint64_t m, uint64_t p) {
+  using namespace imath;
+  const uint32_t mh = hi32(m) & 0x7fffffffu, ph = hi32(p) & 0x7fffffffu;
+  const bool less = pair(mh, lo32(m)) < pair(ph, lo32(p));
+  const uint32_t ah = less ? mh : ph, al = less ? lo32(m) : lo32(p);
+  const uint32_t bh = less ? ph : mh, bl = less ? lo32(p) : lo32(m);
+  const int ea = (int)(ah >> 20), d = (int)(bh >> 20) - ea;
+  const uint32_t fa = (ah & 0xfffffu) | 0x100000u, fb = (bh & 0xfffffu) | 0x100000u;
+  const int n = d < 3 ? d : 3;
+  const uint64_t S = pair(fa, al) + pair(shl_hi(fb, bl, n), bl << n);   // (a + b) 2^(1075 - ea), from 2^53
+  const int top = (int)(hi32(S) >> 22) & 1;                              // S >= 2^54 (below 2^55 where it is taken)
+  const uint32_t lsb = shr_lo(hi32(S), lo32(S), 1 + top) & 1u;
+  const uint64_t r = S + (uint32_t)top + lsb;
+  const uint32_t ch = (hi32(r) >> (1 + top)) + ((uint32_t)(ea - 2 + top) << 20);
+  const uint32_t cl = shr_lo(hi32(r), lo32(r), 1 + top);
+  const bool central = d < 3 && ea > 1 && pair(ch, cl) < pair(ah, al);
+  const bool zero = (int32_t)(hi32(m) ^ hi32(p)) < 0 || (ah | al) == 0;
+  const uint32_t h = (central ? ch : ah) | (hi32(p) & 0x80000000u);
+  return pair(zero ? 0u : h, zero ? 0u : (central ? cl : al));
+}
+
 }  // namespace gbh
