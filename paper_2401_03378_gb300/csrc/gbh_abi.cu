@@ -574,6 +574,7 @@ void layout_from_params(const gbh_params* p, Layout* L, Eos* e) {
     return wide_unpack((uint32_t)(u >> 32), (uint32_t)u);
   };
   e->wgamma = unpacked(e->gamma);
+  e->wgm1 = unpacked(e->gm1);
   e->whgm1 = unpacked(e->hgm1);
   e->wg_gm1 = unpacked(e->g_gm1);
 }

@@ -81,17 +81,8 @@ __device__ __forceinline__ void mc_half_slope_vjp(int br, double bh, double& bqm
 // cons_to_prim reporting which floors applied.
 __device__ __forceinline__ void cons_to_prim_flags(const double U[5], double W[5], const Eos& e, bool& fr,
                                                    bool& fp) {
-  const Rk& k = e.k;
-  double rho = U[0];
-  fr = less_d(rho, e.small_rho);
-  if (fr) rho = e.small_rho;
-  const double ir = rcp_nr(rho, k);
-  const double u = mul(U[1], ir, k), v = mul(U[2], ir, k), w = mul(U[3], ir, k);
-  const double m2 = fma(U[3], w, fma(U[2], v, mul(U[1], u, k)));
-  double p = mul(e.gm1, fma(-half_any(m2), k.one, U[4]), k);
-  fp = less_d(p, e.small_p);
-  if (fp) p = e.small_p;
-  W[0] = rho; W[1] = u; W[2] = v; W[3] = w; W[4] = p;
+  Wide ir;
+  cons_to_prim_flags(U, W, e, ir, fr, fp);
 }
 
 // bU = (dW/dU)^T bW for W = cons_to_prim(U); floored components are constants.

@@ -322,11 +322,13 @@ __global__ void __launch_bounds__(kThreads) reflux_kernel(double* U, const AmrAr
       if (h1 != h0) atomicAdd(a.floor_count, (unsigned long long)(long long)(h1 - h0));
     }
     if (smax_acc) {
-      double W[5], ir;
+      double W[5];
+      Wide ir;
       cons_to_prim_ir(Uc, W, e, ir);
-      const double sp = signal_speed_ir(W, ir, e, reg_const(__ldg(a.inv_dx + 3 * en.block), zt),
-                                        reg_const(__ldg(a.inv_dx + 3 * en.block + 1), zt),
-                                        reg_const(__ldg(a.inv_dx + 3 * en.block + 2), zt), L.ndim == 3);
+      const double ix = reg_const(__ldg(a.inv_dx + 3 * en.block), zt);
+      const double iy = reg_const(__ldg(a.inv_dx + 3 * en.block + 1), zt);
+      const double iz = reg_const(__ldg(a.inv_dx + 3 * en.block + 2), zt);
+      const double sp = signal_speed_ir(W, ir, e, ix, iy, iz, inv_width_sum(e, ix, iy, iz, L.ndim == 3), L.ndim == 3);
       if (a.problem)
         atomicMax(smax_acc + __ldg(a.problem + en.block), (unsigned long long)__double_as_longlong(sp));
       else

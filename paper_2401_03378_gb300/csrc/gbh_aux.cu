@@ -102,12 +102,11 @@ __global__ void __launch_bounds__(kThreads) dt_reduce_kernel(const DtArgs a) {
     double U[5], W[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) U[v] = __ldg(a.U + o + v * L.vstride);
-    double ir;
+    Wide ir;
     cons_to_prim_ir(U, W, e, ir);
-    const double s = signal_speed_ir(W, ir, e, reg_const(__ldg(a.inv_dx + 3 * b), zt),
-                                     reg_const(__ldg(a.inv_dx + 3 * b + 1), zt),
-                                     reg_const(__ldg(a.inv_dx + 3 * b + 2), zt), d3);
-    smax = max_nonneg(smax, s);
+    const double ix = reg_const(__ldg(a.inv_dx + 3 * b), zt), iy = reg_const(__ldg(a.inv_dx + 3 * b + 1), zt);
+    const double iz = reg_const(__ldg(a.inv_dx + 3 * b + 2), zt);
+    smax = max_nonneg(smax, signal_speed_ir(W, ir, e, ix, iy, iz, inv_width_sum(e, ix, iy, iz, d3), d3));
   }
   __shared__ double red[kThreads / 32];
   const double m = block_max<kThreads>(smax, red);
@@ -146,11 +145,11 @@ __global__ void __launch_bounds__(kThreads) dt_reduce_blocks_kernel(const DtArgs
       double U[5], W[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) U[v] = __ldg(a.U + o + v * L.vstride);
-      double ir;
+      Wide ir;
       cons_to_prim_ir(U, W, e, ir);
-      smax = max_nonneg(smax, signal_speed_ir(W, ir, e, reg_const(__ldg(a.inv_dx + 3 * b), zt),
-                                        reg_const(__ldg(a.inv_dx + 3 * b + 1), zt),
-                                        reg_const(__ldg(a.inv_dx + 3 * b + 2), zt), d3));
+      const double ix = reg_const(__ldg(a.inv_dx + 3 * b), zt), iy = reg_const(__ldg(a.inv_dx + 3 * b + 1), zt);
+      const double iz = reg_const(__ldg(a.inv_dx + 3 * b + 2), zt);
+      smax = max_nonneg(smax, signal_speed_ir(W, ir, e, ix, iy, iz, inv_width_sum(e, ix, iy, iz, d3), d3));
     }
     const double m = block_max<kThreads>(smax, red);
     if (threadIdx.x == 0) atomicMax(a.smax_acc + __ldg(problem + b), (unsigned long long)__double_as_longlong(m));
@@ -290,9 +289,10 @@ __global__ void op_count_kernel(int iters, const Eos e0, double* io) {
     } else if constexpr (FN == 4) {   // the second-stage combine of one variable
       fb ^= dbits(half_any(add(x[1], x[0], rk)));
     } else if constexpr (FN == 5) {   // CFL epilogue of one cell: cons -> prim and 3-D signal speed
-      double W[5], ir;
+      double W[5];
+      Wide ir;
       cons_to_prim_ir(x, W, e, ir);
-      fb ^= dbits(signal_speed_ir(W, ir, e, c1, c2, c3, true));
+      fb ^= dbits(signal_speed_ir(W, ir, e, c1, c2, c3, c1, true));
     } else if constexpr (FN == 6) {   // z march: the next z slope and face states of one variable
       const double dn = sub(x[1], x[0], rk);
       const double tz = mc_half_slope_d(x[2], dn, rk);

@@ -30,25 +30,82 @@ __device__ __forceinline__ uint64_t word_pair(double x) {
   return imath::pair((uint32_t)__double2hiint(x), (uint32_t)__double2loint(x));
 }
 
+// Wide -> double, for a result in the normal range.
+__device__ __forceinline__ double wide_double(const Wide& a) { return bitsd((long long)wide_pack(a)); }
+
+__device__ __forceinline__ uint32_t hi_word(double x) { return (uint32_t)((unsigned long long)dbits(x) >> 32); }
+
+// The unpacked magnitude of x, with zeros (and subnormals) as numbers so small
+// that no product of the scheme brings them back into the range of a double.
+__device__ __forceinline__ Wide wide_of0(double x) {
+  Wide a = wide_of(x);
+  a.e = a.e == 0 ? -8192 : a.e;
+  return a;
+}
+
+// Wide -> double with the bits of `top` (a sign bit; a NaN's exponent and
+// quiet bits) OR-ed in: below the normal range a zero, above it an infinity or NaN.
+__device__ __forceinline__ double wide_signed(const Wide& a, uint32_t top) {
+  const uint64_t m = wide_pack(Wide{a.h, a.l, a.e < 2047 ? a.e : 2047});
+  const bool in = a.e >= 1;
+  return bitsd((long long)imath::pair((in ? imath::hi32(m) : 0u) | top, in ? imath::lo32(m) : 0u));
+}
+
+// 0 or 1: the sign of x (as a number, not a masked word: the compiler turns an
+// XOR of masked sign bits into an FP64 negation).
+__device__ __forceinline__ uint32_t sign01(double x) { return hi_word(x) >> 31; }
+
+// Infinity or NaN.
+__device__ __forceinline__ bool not_finite(double x) { return (hi_word(x) & 0x7ff00000u) == 0x7ff00000u; }
+
+// See hllc_flux.
+__device__ __forceinline__ uint32_t non_finite_mask(const double WL[5], const double WR[5]) {
+  float z = 0.0f;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    z = fmaf(__uint_as_float(hi_word(WL[v])), 0.0f, z);
+    z = fmaf(__uint_as_float(hi_word(WR[v])), 0.0f, z);
+  }
+  return __float_as_uint(z);
+}
+
 // calcEos role: conserved (rho, mx, my, mz, E) -> primitive (rho, u, v, w, p),
-// p = (gamma-1) (E - (mx u + my v + mz w)/2).  Floors rho at small_rho and p
-// at small_p; returns 1 when a floor applied.
-__device__ __forceinline__ int cons_to_prim_ir(const double U[5], double W[5], const Eos& e, double& ir) {
-  const Rk& k = e.k;
-  int hit = 0;
+// p = (gamma-1) (E - (mx^2 + my^2 + mz^2) / (2 rho)).  Floors rho at small_rho and
+// p at small_p (floored_rho, floored_p) and leaves 1/rho in ir.  On the integer pipes but
+// for the subtraction: 8 FP64 instructions of 64 cycles became 1 and about 110
+// more integer ones; a NaN or infinity in any of the five reaches u, v, w and p through
+// the FP32 mask.
+__device__ __forceinline__ void cons_to_prim_flags(const double U[5], double W[5], const Eos& e, Wide& ir,
+                                                   bool& floored_rho, bool& floored_p) {
+  float z = 0.0f;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) z = fmaf(__uint_as_float(hi_word(U[v])), 0.0f, z);
+  const uint32_t bad = __float_as_uint(z);
   double rho = U[0];
-  if (less_d(rho, e.small_rho)) { rho = e.small_rho; hit = 1; }
-  ir = rcp_nr(rho, k);
-  const double u = mul(U[1], ir, k), v = mul(U[2], ir, k), w = mul(U[3], ir, k);
-  const double m2 = fma(U[3], w, fma(U[2], v, mul(U[1], u, k)));   // >= 0
-  double p = mul(e.gm1, fma(-half_any(m2), k.one, U[4]), k);       // (gamma-1) (E - m2/2)
-  if (less_d(p, e.small_p)) { p = e.small_p; hit = 1; }
+  floored_rho = less_d(rho, e.small_rho);
+  if (floored_rho) rho = e.small_rho;
+  ir = wide_rcp(wide_of(rho));
+  const Wide mx = wide_of0(U[1]), my = wide_of0(U[2]), mz = wide_of0(U[3]);
+  const double u = wide_signed(wide_mul(mx, ir), sign01(U[1]) << 31 | bad);
+  const double v = wide_signed(wide_mul(my, ir), sign01(U[2]) << 31 | bad);
+  const double w = wide_signed(wide_mul(mz, ir), sign01(U[3]) << 31 | bad);
+  const Wide m2 = wide_mul(wide_add(wide_add(wide_mul(mx, mx), wide_mul(my, my)), wide_mul(mz, mz)), ir);
+  const double ein = sub(U[4], wide_signed(Wide{m2.h, m2.l, m2.e - 1}, 0u), e.k);
+  double p = wide_signed(wide_mul(e.wgm1, wide_of0(ein)), sign01(ein) << 31 | bad);
+  floored_p = less_d(p, e.small_p);
+  if (floored_p) p = e.small_p;
   W[0] = rho; W[1] = u; W[2] = v; W[3] = w; W[4] = p;
-  return hit;
+}
+
+// The same; returns 1 when a floor applied.
+__device__ __forceinline__ int cons_to_prim_ir(const double U[5], double W[5], const Eos& e, Wide& ir) {
+  bool fr, fp;
+  cons_to_prim_flags(U, W, e, ir, fr, fp);
+  return fr || fp ? 1 : 0;
 }
 
 __device__ __forceinline__ int cons_to_prim(const double U[5], double W[5], const Eos& e) {
-  double ir;
+  Wide ir;
   return cons_to_prim_ir(U, W, e, ir);
 }
 
@@ -116,57 +173,19 @@ __device__ __forceinline__ double block_max(double v, double* s_warp) {
   return v;
 }
 
-// Wide -> double, for a result in the normal range.
-__device__ __forceinline__ double wide_double(const Wide& a) { return bitsd((long long)wide_pack(a)); }
-
-__device__ __forceinline__ uint32_t hi_word(double x) { return (uint32_t)((unsigned long long)dbits(x) >> 32); }
-
-// The unpacked magnitude of x, with zeros (and subnormals) as numbers so small
-// that no product of the scheme brings them back into the range of a double.
-__device__ __forceinline__ Wide wide_of0(double x) {
-  Wide a = wide_of(x);
-  a.e = a.e == 0 ? -8192 : a.e;
-  return a;
+// The sum of the inverse cell widths that signal_speed_ir takes, in its order.
+__device__ __forceinline__ double inv_width_sum(const Eos& e, double idx, double idy, double idz, bool dim3) {
+  return dim3 ? add(add(idx, idy, e.k), idz, e.k) : add(idx, idy, e.k);
 }
 
-// Wide -> double with the bits of `top` (a sign bit; a NaN's exponent and
-// quiet bits) OR-ed in: below the normal range a zero, above it an infinity or NaN.
-__device__ __forceinline__ double wide_signed(const Wide& a, uint32_t top) {
-  const uint64_t m = wide_pack(Wide{a.h, a.l, a.e < 2047 ? a.e : 2047});
-  const bool in = a.e >= 1;
-  return bitsd((long long)imath::pair((in ? imath::hi32(m) : 0u) | top, in ? imath::lo32(m) : 0u));
-}
-
-// 0 or 1: the sign of x (as a number, not a masked word: the compiler turns an
-// XOR of masked sign bits into an FP64 negation).
-__device__ __forceinline__ uint32_t sign01(double x) { return hi_word(x) >> 31; }
-
-// a^2 + b^2 + c^2
-__device__ __forceinline__ Wide wide_square_sum(double a, double b, double c) {
-  const Wide x = wide_of(a), y = wide_of(b), z = wide_of(c);
-  return wide_add(wide_add(wide_mul(x, x), wide_mul(y, y)), wide_mul(z, z));
-}
-
-// See hllc_flux.
-__device__ __forceinline__ uint32_t non_finite_mask(const double WL[5], const double WR[5]) {
-  float z = 0.0f;
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    z = fmaf(__uint_as_float(hi_word(WL[v])), 0.0f, z);
-    z = fmaf(__uint_as_float(hi_word(WR[v])), 0.0f, z);
-  }
-  return __float_as_uint(z);
-}
-
-// Signal-speed sum of one cell for the CFL rule; W from cons_to_prim and
-// ir = 1 / W[0] (cons_to_prim_ir returns it).
-__device__ __forceinline__ double signal_speed_ir(const double W[5], double ir, const Eos& e, double idx,
-                                                  double idy, double idz, bool dim3) {
-  const Rk& k = e.k;
-  const double c = sqrt_nr(mul(mul(e.gamma, W[4], k), ir, k), k);
-  // sum_d (|u_d| + c) / dx_d = c (1/dx + 1/dy [+ 1/dz]) + |u| / dx + |v| / dy [+ |w| / dz]
-  const double isum = dim3 ? add(add(idx, idy, k), idz, k) : add(idx, idy, k);
-  double s = fma(fabs(W[1]), idx, mul(c, isum, k));
+// Signal-speed sum of one cell for the CFL rule,
+// sum_d (|u_d| + c) / dx_d = c (1/dx + 1/dy [+ 1/dz]) + |u| / dx + |v| / dy [+ |w| / dz];
+// W and ir = 1 / W[0] from cons_to_prim_ir, isum = inv_width_sum(...).
+__device__ __forceinline__ double signal_speed_ir(const double W[5], const Wide& ir, const Eos& e, double idx,
+                                                  double idy, double idz, double isum, bool dim3) {
+  const Wide c = wide_sqrt(wide_mul(wide_mul(e.wgamma, wide_of(W[4])), ir));
+  const double c_d = not_finite(W[4]) ? W[4] : wide_double(c);
+  double s = fma(fabs(W[1]), idx, mul(c_d, isum, e.k));
   s = fma(fabs(W[2]), idy, s);
   if (dim3) s = fma(fabs(W[3]), idz, s);
   return s;
@@ -209,9 +228,12 @@ __device__ __forceinline__ double signal_speed_ir(const double W[5], double ir, 
 // instructions a face with the remaining roots and reciprocals; of that the
 // chain: 256^3 step 16.71 -> 14.07 ms, 96-problem 2-D ensemble 6.88 -> 5.71 ms.
 // The quotients S* and t, whose factors are already unpacked, follow the same
-// way (m_L - m_R is a sum of two negative numbers), as do the other products and
-// the sums of squares: 19 FP64 instructions a face are left, the differences
-// and the sums of numbers of either sign (256^3 step 14.07 -> 13.39 -> 12.33 ms).
+// way (m_L - m_R is a sum of two negative numbers), as do m_K, h_K, rho_K t and
+// g m_K: 26 FP64 instructions a face are left (256^3 step 14.07 -> 12.33 ms).  The
+// sums of squares and the products with v_K and w_K stay on the FP64 pipe: a
+// face takes about 1050 integer instructions, and with these eight in integer
+// form too (19 FP64, 1150) the integer pipes were the longer ones inside the
+// face passes (96-problem ensemble 4.89 -> 4.73 ms, 256^3 11.74 -> 11.62 ms).
 __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5], const Eos& e,
                                           double F[5]) {
   const Rk& k = e.k;
@@ -235,7 +257,7 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
 
   const double du = sub(uL, uR, k), dv = sub(vL, vR, k), dw = sub(wL, wR, k);
   const double ut = fma(-wide_double(wr), du, uL);         // w_L u_L + w_R u_R
-  const Wide du2 = wide_square_sum(du, dv, dw);
+  const Wide du2 = wide_of(fma(dw, dw, fma(dv, dv, mul(du, du, k))));
   const Wide ct2 = wide_add(wide_mul(wl, cL2),
                             wide_mul(wr, wide_add(cR2, wide_mul(wide_mul(e.whgm1, wl), du2))));
   const double ct = wide_double(wide_sqrt(ct2));
@@ -265,17 +287,17 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
   const uint32_t tsgn = fan ? ssgn ^ sign01(SKs) ^ (left ? 1u : 0u) : sign01(uK);
   const double t = wide_signed(T, tsgn << 31 | bad);
   const double g = sub(t, uK, k);
-  const Wide RK = wide_of(rK), VK = wide_of0(vK), WK = wide_of0(wK);
+  const Wide RK = wide_of(rK);
   // E + p of the chosen side
-  const Wide kin = wide_mul(RK, wide_square_sum(uK, vK, wK));
+  const Wide kin = wide_mul(RK, wide_of(fma(wK, wK, fma(vK, vK, mul(uK, uK, k)))));
   const double hK = wide_double(wide_add(Wide{kin.h, kin.l, kin.e - 1}, wide_mul(e.wg_gm1, wide_of(pK))));
   const Wide F0 = wide_mul(RK, T);
   const Wide GM = wide_mul(wide_of0(g), left ? ML : MR);   // |g m_K|
   const uint32_t gmsgn = sign01(g) ^ (left ? 1u : 0u);
   F[0] = wide_signed(F0, tsgn << 31 | bad);
   F[1] = add(fma(F[0], uK, pK), wide_signed(GM, gmsgn << 31), k);
-  F[2] = wide_signed(wide_mul(VK, F0), (sign01(vK) ^ tsgn) << 31 | bad);
-  F[3] = wide_signed(wide_mul(WK, F0), (sign01(wK) ^ tsgn) << 31 | bad);
+  F[2] = mul(vK, F[0], k);
+  F[3] = mul(wK, F[0], k);
   F[4] = fma(hK, t, wide_signed(wide_mul(GM, WS), (gmsgn ^ ssgn) << 31));
 }
 

@@ -34,8 +34,8 @@ struct Eos {
   double gamma, gm1, inv_gm1, g_gm1, small_rho, small_p;  // g_gm1 = gamma / (gamma - 1)
   double hgm1;                                            // (gamma - 1) / 2
   Rk k;                                                   // {1, -0}
-  Wide wgamma, whgm1, wg_gm1;                             // gamma, (gamma - 1) / 2 and gamma / (gamma - 1)
-                                                          // unpacked (gbh_intmath.cuh)
+  Wide wgamma, wgm1, whgm1, wg_gm1;                       // gamma, gamma - 1, (gamma - 1) / 2 and
+                                                          // gamma / (gamma - 1) unpacked (gbh_intmath.cuh)
   long long opaque;                                       // 0 (see reg_eos)
 };
 

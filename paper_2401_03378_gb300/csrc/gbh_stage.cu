@@ -158,13 +158,14 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
   const long long zt = thread_zero(a.eos);
   const Eos e = reg_eos(a.eos, zt);
   const Rk& rk = e.k;
-  // dt/dx, dt/dy, dt/dz: formed once per item by thread 0 and read back in
-  // the update, after the plane's barriers (three FP64 multiplies per thread
-  // otherwise, which an item of one 2-D plane pays per cell)
+  // dt/dx, dt/dy, dt/dz and 1/dx + 1/dy + 1/dz: formed once per item by thread
+  // 0 and read back in the update, after the plane's barriers (five FP64
+  // operations per thread otherwise, which an item of one 2-D plane pays per cell)
   if (tid == 0) {
     s_dt[0] = dt * idx;
     s_dt[1] = dt * idy;
     s_dt[2] = DIM3 ? dt * idz : 0.0;
+    s_dt[3] = inv_width_sum(e, idx, idy, idz, DIM3);
   }
 
   int hits = 0;
@@ -544,7 +545,8 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
     }
     if (E == 0 && (a.smax_acc || a.Wout)) {
       // calcEos of the new state: the CFL speed, and the next stage's primitives
-      double W[5], ir;
+      double W[5];
+      Wide ir;
       const int h = cons_to_prim_ir(out, W, e, ir);
       if (a.Wout) {
 #pragma unroll
@@ -552,7 +554,8 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
         hits += h;
       }
       if (a.smax_acc) {
-        const double sp = signal_speed_ir(W, ir, e, reg_const(idx, zt), reg_const(idy, zt), reg_const(idz, zt), DIM3);
+        const double sp = signal_speed_ir(W, ir, e, reg_const(idx, zt), reg_const(idy, zt), reg_const(idz, zt),
+                                          reg_const(s_dt[3], zt), DIM3);
         if (!corrected_cell<N, DIM3>(a, b, ci, cj, k, L.nz)) smax = max_nonneg(smax, sp);
       }
     }
@@ -664,7 +667,7 @@ __global__ void __launch_bounds__(stage_threads<N, E, S>(), min_ctas<N, E, S>())
   constexpr int NT = stage_threads<N, E, S>();
   extern __shared__ double smem[];
   __shared__ double s_red[E == 0 && NT > 32 ? NT / 32 : 1];
-  __shared__ double s_dt[3];
+  __shared__ double s_dt[4];
   const int nitems = (a.block_list ? a.nlist : a.lay.nblocks) * a.nchunks * S;
   const int first = blockIdx.x * a.items_per_cta;
   const int last = min(nitems, first + a.items_per_cta);
