@@ -447,9 +447,7 @@ gbh::DtArgs dt_args(gbh_ctx* c, const double* U) {
 
 // CFL time step(s) of U into dt_dev (one per problem) and, if given, hist.
 int reduce_dt(gbh_ctx* c, const double* U, double* dt_dev, double* hist, cudaStream_t s) {
-  cudaError_t e = c->d_problem ? gbh::launch_dt_reduce_blocks(dt_args(c, U), c->d_problem, s)
-                               : gbh::launch_dt_reduce(dt_args(c, U), s);
-  int rc = cuda_err(c, e, "dt reduce launch");
+  int rc = cuda_err(c, gbh::launch_dt_reduce(dt_args(c, U), c->d_problem, s), "dt reduce launch");
   if (rc) return rc;
   return cuda_err(c, gbh::launch_dt_finalize(c->d_smax, c->cfl, dt_dev, hist, s, c->nproblems),
                   "dt finalize launch");

@@ -162,10 +162,10 @@ struct DtArgs {
   const int* block_list;   // blocks to include (null = all)
   int nlist;
 };
-cudaError_t launch_dt_reduce(const DtArgs& a, cudaStream_t s);
+// problem: null, or [nblocks] the accumulator of smax_acc each block goes to
+cudaError_t launch_dt_reduce(const DtArgs& a, const int* problem, cudaStream_t s);
 cudaError_t launch_dt_finalize(unsigned long long* acc, double cfl, double* dt_out, double* hist,
                                cudaStream_t s, int n = 1);
-cudaError_t launch_dt_reduce_blocks(const DtArgs& a, const int* problem, cudaStream_t s);
 
 cudaError_t launch_check(const double* U, Layout lay, Eos eos, unsigned long long* count,
                          cudaStream_t s);
