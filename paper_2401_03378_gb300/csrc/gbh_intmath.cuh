@@ -12,8 +12,9 @@
 // once at their end.
 //
 // Wide: a positive number as a 63-bit mantissa and an exponent,
-//     value = (h 2^32 + l) 2^(e - 1023 - 62),  2^62 <= h 2^32 + l < 2^63
-// (results may reach 2^63 itself), e in the biased form of a double.  Products,
+//     value = (h 2^32 + l) 2^(e - 1023 - 62),  2^62 <= h 2^32 + l < 2^63,
+// e in the biased form of a double; a reciprocal, a root or a product of them may
+// be up to 64 units below 2^62, which products, sums, roots and the rounding take.  Products,
 // reciprocals and roots are computed to a relative error below 2^-58 (stated at
 // each), so a double rounded from a chain of them (wide_pack, to nearest) is
 // within 0.55 ulp of the exact value: tighter than the same chain of FP64
@@ -160,7 +161,8 @@ GBH_HD Wide wide_add(const Wide& a, const Wide& b) {
   return r;
 }
 
-// 1 / a: relative error below 2^-58.5.
+// 1 / a: relative error below 2^-58.5.  a is at least 2^62: unpacked, a product
+// of unpacked numbers, or a sum with one of them.
 GBH_HD Wide wide_rcp(const Wide& a) {
   using namespace imath;
   // seed: R0 = 1/f in units of 2^-31, f in [1, 2) the leading 24 bits of a; n0 = -R0
@@ -171,7 +173,7 @@ GBH_HD Wide wide_rcp(const Wide& a) {
   const int32_t e0 = (int32_t)shr_lo(hi32(p0), lo32(p0), 12);
   // R1 = R0 (1 + e0): relative error below 2^-29.4, R1 <= 2^31
   const int32_t x = (int32_t)hi32((uint64_t)muls(n0, e0));
-  const uint32_t r1 = (uint32_t)(-(n0 + (x >> 17)));
+  const uint32_t r1 = 0u - ((uint32_t)n0 + (uint32_t)(x >> 17));
   // E = a R1 - 1 in units of 2^-61 (|E| < 2^32), c = R1 E in units of 2^-60;
   // the signed reading of r1 = 2^31 is harmless: then 0 <= E < 2^32
   const uint64_t E = mulu(a.h, r1) + pair(0xe0000000u, hi32(mulu(a.l, r1)));
@@ -190,7 +192,9 @@ GBH_HD Wide wide_sqrt(const Wide& a) {
   const int odd = ~a.e & 1;                                  // 2^odd m in [1, 4) has an even exponent
   const uint32_t H = shl_hi(a.h, a.l, odd), L = a.l << odd;   // in units of 2^-62
   // seed: R0 = 1/sqrt(f) in units of 2^-31, below 2^31
-  const uint32_t rb = bits_of(rsqrt_seed(float_of((a.h >> 7) + 0x3f000000u + ((uint32_t)odd << 23))));
+  // (from f >= 1: a product or root a few units below 2^62 is taken there)
+  const uint32_t hs = a.h > 0x40000000u ? a.h : 0x40000000u;
+  const uint32_t rb = bits_of(rsqrt_seed(float_of((hs >> 7) + 0x3f000000u + ((uint32_t)odd << 23))));
   const uint32_t r0 = (rb - 0x3e800001u) * 128u;
   // R0^2 in units of 2^-32 (rounded); d0 = H R0^2 - 1 in units of 2^-49
   const uint64_t q = mulu(r0, r0) + (1u << 29);
