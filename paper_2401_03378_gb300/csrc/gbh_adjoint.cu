@@ -44,18 +44,17 @@ namespace {
 // constants of reg_eos in per-thread registers: the same results as the plain
 // operations at the FP64 pipe's full issue rate.
 
-// mc_half_slope with the branch it takes: 0 zero, 1 central, 2 |dm|, 3 |dp|.
+// The half slope of mc_half_slope_d with the branch it takes: 0 zero, 1 central,
+// 2 |dm|, 3 |dp|.
 __device__ __forceinline__ double mc_half_slope_br(double qm, double q0, double qp, int& br, const Rk& k) {
   const double dm = sub(q0, qm, k);
   const double dp = sub(qp, q0, k);
-  const double s4 = quarter_any(add(dm, dp, k));
-  const unsigned long long am = mag_key(dm), ap = mag_key(dp), as = mag_key(s4);
-  const unsigned long long m1 = am < ap ? am : ap;
-  const bool central = as < m1;
-  const unsigned long long m = central ? as : m1;
-  const bool same = ((dbits(dm) ^ dbits(dp)) >= 0) && am != 0 && ap != 0;
-  br = !same ? 0 : (central ? 1 : (am < ap ? 2 : 3));
-  return bitsd(same ? (long long)((m >> 1) | sign_bit(dp)) : 0LL);
+  const uint64_t m = word_pair(dm), p = word_pair(dp);
+  const uint64_t h = half_slope(m, p);
+  const uint64_t am = m << 1, ap = p << 1, as = h << 1;
+  const bool same = as != 0;
+  br = !same ? 0 : (as < (am < ap ? am : ap) ? 1 : (am < ap ? 2 : 3));
+  return bitsd((long long)h);
 }
 
 // Adjoint of mc_half_slope_br's result scaled by SIGN (+1 or -1): the
@@ -102,9 +101,7 @@ __device__ __forceinline__ void prim_vjp(const double W[5], bool fr, bool fp, co
 }
 
 // Reverse of hllc_flux (gbh_device.cuh): the forward is recomputed from the
-// same formulas, grouped for the reverse sweep (one reciprocal square root of
-// rho_L rho_R, the Roe sound speed from w_L c_L^2 + w_R c_R^2 + (gamma-1)/2
-// w_L w_R |u_L - u_R|^2, the star state through t = u_K + g), then
+// same formulas, grouped for the reverse sweep, then
 // (dF/dW)^T bF is accumulated step by step in reverse.  Branches (the min / max of the wave-speed bounds, the side K,
 // the fan) keep the forward's decisions and are taken by selects.
 __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double WR[5], const Eos& e, const double bF[5],
@@ -116,41 +113,63 @@ __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double W
   const double rL = WL[0], uL = WL[1], vL = WL[2], wL = WL[3], pL = WL[4];
   const double rR = WR[0], uR = WR[1], vR = WR[2], wR = WR[3], pR = WR[4];
   // ---- forward ----
-  const double q = rsqrt_nr(M(rL, rR), k);                 // 1/sqrt(rho_L rho_R)
-  const double q2 = M(q, q);
-  const double iL = M(rR, q2), iR = M(rL, q2);             // 1/rho
-  const double gpL = M(e.gamma, pL), gpR = M(e.gamma, pR);
-  const double cL2 = M(gpL, iL), cR2 = M(gpR, iR);         // c^2
-  const double qL = rsqrt_nr(cL2, k), qR = rsqrt_nr(cR2, k);   // 1/c
-  const double cL = M(cL2, qL), cR = M(cR2, qR);
-  const double r = M(rR, q);                               // sqrt(rho_R / rho_L)
-  const double wl = rcp_nr(A(r, k.one), k), wr = M(r, wl);
+  // From the densities and pressures to the sound speeds and Roe weights, and
+  // the quotients S* and t, as in hllc_flux: Wide numbers on the integer pipes.
+  const uint32_t bad = non_finite_mask(WL, WR);
+  const Wide RL = wide_of(rL), RR = wide_of(rR);
+  const Wide P = wide_mul(RL, RR), iP = wide_rcp(P), sP = wide_sqrt(P);
+  const Wide GPL = wide_mul(e.wgamma, wide_of(pL)), GPR = wide_mul(e.wgamma, wide_of(pR));
+  const Wide IL = wide_mul(RR, iP), IR = wide_mul(RL, iP);   // 1/rho
+  const Wide CL2 = wide_mul(GPL, IL), CR2 = wide_mul(GPR, IR);
+  const Wide CL = wide_sqrt(CL2), CR = wide_sqrt(CR2);
+  const Wide Q = wide_mul(sP, iP);                           // 1/sqrt(rho_L rho_R)
+  const Wide D = wide_rcp(wide_add(sP, RR));
+  const Wide XL = wide_mul(sP, D), XR = wide_mul(RR, D);     // Roe weights
+  const double q = wide_double(Q), q2 = wide_double(iP);
+  const double iL = wide_double(IL), iR = wide_double(IR);
+  const double gpL = wide_double(GPL), gpR = wide_double(GPR);
+  const double cL2 = wide_double(CL2), cR2 = wide_double(CR2);
+  const double cL = wide_double(CL), cR = wide_double(CR);
+  const double qL = wide_double(wide_rcp(wide_of(cL))), qR = wide_double(wide_rcp(wide_of(cR)));   // 1/c
+  const double r = wide_double(wide_mul(RR, Q));             // sqrt(rho_R / rho_L)
+  const double wl = wide_double(XL), wr = wide_double(XR);
   const double ut = fma(wl, uL, M(wr, uR));
   const double du = S(uL, uR), dv = S(vL, vR), dw = S(wL, wR);
   const double du2 = fma(dw, dw, fma(dv, dv, M(du, du)));
-  const double Bw = M(e.hgm1, M(wl, wr));
-  const double ct2 = fma(Bw, du2, fma(wl, cL2, M(wr, cR2)));
-  const double qc = rsqrt_nr(ct2, k);
-  const double ct = M(ct2, qc);
+  const Wide BW = wide_mul(wide_mul(e.whgm1, XL), XR);
+  const double Bw = wide_double(BW);
+  const Wide CT = wide_sqrt(wide_add(wide_add(wide_mul(XL, CL2), wide_mul(XR, CR2)), wide_mul(BW, wide_of(du2))));
+  const double ct = wide_double(CT), qc = wide_double(wide_rcp(wide_of(ct)));
   const double l1 = S(uL, cL), l2 = S(ut, ct), r1 = A(uR, cR), r2 = A(ut, ct);
   const bool selL1 = !(order_key(l2) < order_key(l1));     // S_L = l1
   const bool selR1 = !(order_key(r1) < order_key(r2));     // S_R = r1
   const double SL = selL1 ? l1 : l2, SR = selR1 ? r1 : r2;
   const double dL = S(SL, uL), dR = S(SR, uR);
-  const double mL = M(rL, dL), mR = M(rR, dR);
-  const double rd = rcp_nr(S(mL, mR), k);
-  const double Ss = M(fma(-mR, uR, fma(mL, uL, S(pR, pL))), rd);
+  const Wide DL = wide_of0(dL), DR = wide_of0(dR);
+  const Wide ML = wide_mul(RL, DL), MR = wide_mul(RR, DR);
+  const double mL = wide_signed(ML, 0x80000000u), mR = wide_signed(MR, 0u);
+  const Wide RD = wide_rcp(wide_add(ML, MR));              // -1 / (mL - mR)
+  const double rd = wide_signed(RD, 0x80000000u);
+  const double num = fma(-mR, uR, fma(mL, uL, S(pR, pL)));
+  const Wide WS = wide_mul(wide_of0(num), RD);
+  const uint32_t ssgn = sign01(num) ^ 1u;
+  const double Ss = wide_signed(WS, ssgn << 31 | bad);
   const bool left = ge0(Ss);
   const double rK = sel(left, rL, rR), uK = sel(left, uL, uR), vK = sel(left, vL, vR);
   const double wK = sel(left, wL, wR), pK = sel(left, pL, pR);
   const double SK = sel(left, SL, SR), mK = sel(left, mL, mR), dK = sel(left, dL, dR);
   const bool fan = left ? lt0(SL) : gt0(SR);
-  const double R = rcp_nr(S(SK, Ss), k);                   // used inside the fan only
-  const double dKR = M(dK, R);
-  const double t = sel(fan, M(Ss, dKR), uK);
+  const double SKs = S(SK, Ss);
+  const Wide WR1 = wide_rcp(wide_of(SKs));                 // used inside the fan only
+  const Wide DKR = wide_mul(left ? DL : DR, WR1);
+  const uint32_t rsgn = sign01(SKs), dsgn = rsgn ^ (left ? 1u : 0u);
+  const double R = wide_signed(WR1, rsgn << 31);
+  const double dKR = wide_signed(DKR, dsgn << 31);
+  const double t = sel(fan, wide_signed(wide_mul(WS, DKR), (ssgn ^ dsgn) << 31 | bad), uK);
   const double g = S(t, uK);
   const double kK = fma(wK, wK, fma(vK, vK, M(uK, uK)));
-  const double hK = fma(half_pos(rK), kK, M(e.g_gm1, pK));
+  const Wide RK = wide_of(rK), KIN = wide_mul(RK, wide_of(kK));
+  const double hK = wide_double(wide_add(Wide{KIN.h, KIN.l, KIN.e - 1}, wide_mul(e.wg_gm1, wide_of(pK))));
   const double gm = M(g, mK);
   const double F0 = M(rK, t);
   // ---- reverse ----
@@ -447,10 +466,20 @@ __global__ void vjp_prim_padded_kernel(const StageArgs a, double* __restrict__ W
 __device__ __forceinline__ void add_position(const FaceGeom& G, const double* __restrict__ C, int d, int b, int pen,
                                              int q, double acc[5], const Rk& kr) {
   const int nd = G.n[d];
-  for (int k = q - 1; k <= q + 2; ++k) {
-    if (k < 0 || k > nd) continue;
-    const double* c = C + slot_index(G, d, b, pen, k, q + 2 - k);
-    for (int v = 0; v < 5; ++v) acc[v] = add(acc[v], c[v], kr);
+  // the loads of the four faces go out together, before the first sum
+  double c[4][5];
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int k = q - 1 + s;
+    const double* p = C + slot_index(G, d, b, pen, k < 0 ? 0 : k > nd ? nd : k, 3 - s);
+#pragma unroll
+    for (int v = 0; v < 5; ++v) c[s][v] = __ldg(p + v);
+  }
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    if (q - 1 + s < 0 || q - 1 + s > nd) continue;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) acc[v] = add(acc[v], c[s][v], kr);
   }
 }
 

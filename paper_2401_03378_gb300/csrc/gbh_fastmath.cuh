@@ -7,14 +7,7 @@
 //    instructions of 64 issue cycles each; 29 of the 80 a face needs.  3-D step
 //    of 256^3: 20.88 -> 16.71 ms, of 128^3: 3.105 -> 2.495 ms, 96-problem 2-D
 //    ensemble 8.52 -> 6.88 ms.
-//  * the reciprocal square root (the adjoint's) starts from the hardware's
-//    documented approximation (PTX rsqrt.approx.ftz.f64) and is refined by ONE
-//    third-order series step (the classical iteration, see e.g. Muller et al.,
-//    Handbook of Floating-Point Arithmetic, ch. 5): with e = 1 - x y0^2,
-//        1/sqrt(x) = y0 (1 + e/2 + 3 e^2/8 + ...),
-//    truncated after the quadratic term, so the relative error of the seed
-//    is cubed; within a few ulp of the correctly rounded result.
-//    All three take positive (the reciprocal: also negative), normal, finite
+//    All take positive (the reciprocal: also negative), normal, finite
 //    inputs -- what the scheme feeds them.
 //  * comparisons, min / max and sign tests of doubles are done on the bit
 //    patterns with 64-bit integer operations (ALU pipe), which give the same
@@ -96,12 +89,6 @@ __device__ __forceinline__ double quarter_any(double x) {
   return bitsd(m2 >= (6ULL << 52) ? dbits(x) - (2LL << 52) : (long long)(sign_bit(x) | (m2 >> 3)));
 }
 
-__device__ __forceinline__ double rsqrt_approx(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-
 // The unpacked magnitude of x, and x from a bit pattern held as two words.
 __device__ __forceinline__ Wide wide_of(double x) {
   return wide_unpack((uint32_t)((unsigned long long)dbits(x) >> 32), (uint32_t)dbits(x));
@@ -116,21 +103,6 @@ __device__ __forceinline__ double rcp_nr(double x) {
 }
 __device__ __forceinline__ double rcp_nr(double x, const Rk&) { return rcp_nr(x); }
 
-// The series term e/2 + 3e^2/8 of the square-root refinements, as h + (3/2) h^2
-// with h = e/2 (exponent decrement on the integer pipe): 2 FP64 operations.
-__device__ __forceinline__ double rsqrt_corr(double e, const Rk& k) {
-  const double h = half_any(e);
-  return fma(add(h, half_any(h), k), h, h);
-}
-
-// 1/sqrt(x): 5 FP64 operations after the seed.
-__device__ __forceinline__ double rsqrt_nr(double x, const Rk& k) {
-  const double y = rsqrt_approx(x);
-  const double t = mul(x, y, k);
-  const double e = fma(-t, y, k.one);
-  return fma(y, rsqrt_corr(e, k), y);
-}
-
 // sqrt(x) on the integer pipes (gbh_intmath.cuh), within 0.56 ulp: no FP64
 // operation (5 before).  NaN for zeros, subnormals, negative values, infinities and NaN.
 __device__ __forceinline__ double sqrt_nr(double x) {
@@ -140,7 +112,8 @@ __device__ __forceinline__ double sqrt_nr(double x) {
 }
 __device__ __forceinline__ double sqrt_nr(double x, const Rk&) { return sqrt_nr(x); }
 
-__device__ __forceinline__ double rsqrt_nr(double x) { return rsqrt_nr(x, plain_rk()); }
+// 1/sqrt(x) as the rounded root's reciprocal, the form the adjoint's 1/c takes.
+__device__ __forceinline__ double rsqrt_nr(double x) { return rcp_nr(sqrt_nr(x)); }
 
 // ---- integer-domain comparisons -------------------------------------------
 
