@@ -201,6 +201,22 @@ int auto_kchunk(int span, long long nblk, int threads, int sms) {
   return best;
 }
 
+// Whether an interior stage of `items` whole-width work items runs with a thread
+// per face (StageArgs::wide; blocks of 16 then in two row bands).  With few items
+// the time of a stage is the chain of one CTA: its slopes of five variables and two
+// passes of faces one after another.  Us per step (two stages), before and with
+// wide CTAs: 2-D, 64 blocks of 16^2 37.0 -> 28.8 (the two bands need 2 items / SM: at
+// 144 blocks 36.0 and 47.8); 91 blocks of 8^2 39.0 -> 26.7, 400: 43.1 -> 32.9, 512: 44.2
+// and 46.2; blocks of 4^2 (half a warp of columns) 91: 41.1 -> 24.6, 4096: 111.8 ->
+// 91.7.  3-D, 4 blocks of 16^3 (64 items) 67.6 -> 47.5; 8 of 8^3 (64 items) 68.0 ->
+// 43.3, 27 (216 items) 68.0 and 76.0; 64 of 4^3 (256 items) 68.0 -> 43.4, 512 (2048
+// items) 98.8 and 149.2.
+bool take_wide(int nx, bool dim3, long long items, int sms) {
+  if (nx == 16) return 2 * items <= sms;
+  if (nx == 8) return items <= (dim3 ? 1 : 3) * (long long)sms;
+  return !dim3 || items <= 2LL * sms;
+}
+
 // One stage launch.  ring > 0: the telescoping form that also updates that
 // many guard cells around the interior, from Uin's own guard cells.
 // range_first >= 0: `list` is the identity list of blocks [range_first,
@@ -248,6 +264,12 @@ int stage_launch(gbh_ctx* c, const double* Uin, const double* Un, double* Uout, 
                                                               : auto_kchunk(span, nblk, side * side / A.ysplit, c->sms);
     A.kchunk = k > 0 ? k : span;
     A.nchunks = (span + A.kchunk - 1) / A.kchunk;
+  }
+  const long long items = (list ? nlist : c->refined ? c->nactive : c->lay.nblocks) * (long long)A.nchunks;
+  if (c->kchunk < 0 && ring == 0 && A.ysplit == 1 && !(prepass && A.nchunks == 1) &&
+      take_wide(c->lay.nx, c->lay.ndim == 3, items, c->sms)) {
+    A.wide = 1;
+    if (c->lay.nx == 16) A.ysplit = 2;
   }
   A.items_per_cta = c->items_per_cta;
   if (c->refined) {
@@ -599,6 +621,7 @@ void stage_args_common(StageArgs* A, const Layout& L, const Eos& e) {
   A->nchunks = 1;
   A->items_per_cta = 1;
   A->ysplit = 1;
+  A->wide = 0;
 }
 
 int set_create_error(int code, const char* msg) { return set_err(nullptr, code, "%s", msg); }
@@ -981,7 +1004,15 @@ int gbh_autotune(gbh_ctx* c, const double* U, int* kchunk_out, int* items_out, v
   // keeps two CTAs per SM resident, a band four)
   float best = 1e30f;
   int best_kc = 0, best_ipc = 1, best_split = 1;
+  if (c->lay.ndim == 2) {
+    // first what a launch chooses by itself (wide CTAs on a small lattice)
+    best_kc = c->kchunk = -1;
+    c->items_per_cta = 1;
+    c->ysplit[0] = 1;
+    rc = time_stage(c, U, 0, e0, e1, s, &best);
+  }
   for (int split : splits) {
+    if (rc) break;
     for (int kc : kcs) {
       const long long nitems = nlist * (kc > 0 ? (c->lay.nz + kc - 1) / kc : 1) * split;
       const long long resident = 2LL * split * sms;

@@ -54,6 +54,7 @@ struct StageArgs {
   int kchunk, nchunks;   // z planes per work item (3-D), work items per block
   int items_per_cta;     // consecutive work items processed by one CTA (>= 1)
   int ysplit;            // row bands per plane tile, one CTA each (1, or 2 for nx >= 8)
+  int wide;              // interior stages without the pre-pass: 1 = a thread per face of the band
   const int* problem;    // [nblocks] problem of each block (batched ensembles), or null
                          // (then dt_dev and smax_acc have one entry)
   Layout lay;

@@ -89,17 +89,41 @@ constexpr int stage_threads() {
   return E == 2 && S == 1 ? N * (N + 4 * E) : (N + 2 * E) * (N + 2 * E) / S;
 }
 
+// Threads of a wide CTA: one per face of a plane (all x and y faces of the band,
+// its upper boundary included), in whole warps.
+template <int N, int S>
+constexpr int wide_threads() {
+  return (N / S * (N + 1) + (N / S + 1) * N + 31) / 32 * 32;
+}
+
+// Row bands of a wide launch.
+template <int N>
+constexpr int wide_bands() { return N == 16 ? 2 : 1; }
+
+template <int N, int E, int S, bool WIDE>
+constexpr int cta_threads() { return WIDE ? wide_threads<N, S>() : stage_threads<N, E, S>(); }
+
 // One work item: block `b` of the list (or of the lattice), z-chunk `chunk`
 // and row band `band` of the plane tile.  The (N+2E)-wide plane tile is cut
 // into S bands of MY = (N+2E)/S rows; a CTA of M*MY threads updates one band
 // (S = 1: the whole tile).  Uses the caller's shared memory; ends with the
 // per-item atomics.
-template <int N, bool DIM3, int E, int S, bool BF = false>
+//
+// WIDE (interior stages): more threads than columns, for lattices with too few
+// work items to fill the chip, where the time of an item is the length of one
+// thread's chain and not the throughput of the SM.  Every face of the plane gets a
+// thread of its own in (C), the band's upper boundary faces among them (from the
+// slope list's face states, the same arithmetic on the same values), and the slope
+// list is cut into (item, variable) pairs; the threads past the columns take part
+// in the lists only.
+template <int N, bool DIM3, int E, int S, bool BF = false, bool WIDE = false>
 __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double* smem, double* s_red,
                                            double* s_dt) {
   constexpr int M = N + 2 * E;              // plane tile width (the interior when E = 0)
   constexpr int MY = M / S;                 // rows of one band
-  constexpr int NT = stage_threads<N, E, S>();   // threads: one per updated column
+  constexpr int NCOL = stage_threads<N, E, S>(); // updated columns, one thread each
+  constexpr int NT = cta_threads<N, E, S, WIDE>();
+  static_assert(!WIDE || (E == 0 && !BF), "wide CTAs run interior stages without the pre-pass");
   constexpr int PX = M + 4, PY = MY + 4;    // band with 2-deep x/y rims
   constexpr int QXS = MY * (M + 2);         // x face states of a band, per variable and side
   constexpr int QYS = (MY + 2) * M;         // y face states
@@ -141,6 +165,8 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
   } else {
     tx = tid % M; ty = tid / M;
   }
+  const bool col = !WIDE || tid < NCOL;     // this thread updates a column
+  if (!col) tx = ty = 0;
   const int ci = tx - E, cj = y0 + ty - E;
   const int slot_idx = rest / a.nchunks;
   const int chunk = rest - slot_idx * a.nchunks;
@@ -181,7 +207,7 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
   // have N nz, z faces N N), N in 2-D
   const int NF = DIM3 ? N * (L.nz > N ? L.nz : N) : N;
   const double* bfb = bf ? a.bflux + (long long)b * 6 * 5 * NF : nullptr;
-  if (DIM3) {
+  if (DIM3 && col) {
     double Wm2[5], Wm1[5], qpm1[5], qm0[5];
     constexpr bool bottom = bf;                // the z face -1/2 comes from the pre-pass
     if (!bottom) stage_prim<N, E>(a, e, b, ci, cj, k0 - 2, Wm2);
@@ -210,14 +236,14 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
       hllc_flux(wl, wr, e, f);
       Fzm[0] = f[0]; Fzm[1] = f[2]; Fzm[2] = f[3]; Fzm[3] = f[1]; Fzm[4] = f[4];
     }
-  } else {
+  } else if (!DIM3 && col) {
     const int h0 = stage_prim<N, E>(a, e, b, ci, cj, 0, W0);
     if (col_in) hits += h0;
   }
 
   for (int k = k0; k < k1; ++k) {
     double Fzp[5], Wn[5], qpn[5];
-    if constexpr (E == 0) {
+    if (E == 0 && col) {
       // Into L1 ahead of their use: the conserved operands of this plane's
       // update (D), which nothing else reads when the primitives come from
       // a.Win, and the z march's cell of the next iteration (plane k + 3 of
@@ -241,7 +267,7 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
       // the z face nz - 1/2 comes from the pre-pass
 #pragma unroll
       for (int v = 0; v < 5; ++v) Fzp[v] = bfb[(FACE_ZP * 5 + v) * NF + cj * N + ci];
-    } else if (DIM3) {
+    } else if (DIM3 && col) {
       // own column: primitives at k+2, face states of k+1, z flux at k + 1/2
       const int hn = stage_prim<N, E>(a, e, b, ci, cj, k + 2, Wn);
       if (counted(k + 2)) hits += hn;
@@ -282,8 +308,10 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
 
     // (A) primitives of plane k in the band and its 2-deep x/y rims -> shared
     //     memory (i, j: band positions)
+    if (col) {
 #pragma unroll
-    for (int v = 0; v < 5; ++v) sW[GBH_IX((v * PY + ty + 2) * PX + tx + 2, 5 * PY * PX)] = W0[v];
+      for (int v = 0; v < 5; ++v) sW[GBH_IX((v * PY + ty + 2) * PX + tx + 2, 5 * PY * PX)] = W0[v];
+    }
     if constexpr (S == 1) {
       // the whole tile: all four rims (and at ring 2 the 16 cells of the
       // corner columns, which have no thread) on every plane except the
@@ -361,7 +389,43 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
     const bool trim = E == 2 && S == 1 && !outer;
     const int TRX = (Wx + 4) / 3, TRY = (Wy + 4) / 3;   // triples per line (W + 2 slope cells)
     const int NSX = TRX * Wy, NSY = TRY * Wx;
-    for (int s = rtid; s < NSX + NSY + (bf ? 2 : 1) * (Wy + Wx); s += NT) {
+    // one variable of one slope item
+    auto slopes = [&](int s, int v) {
+      const bool xs = s < NSX;
+      const int s2 = xs ? s : s - NSX;
+      const int TR = xs ? TRX : TRY, Wl = xs ? Wx : Wy;
+      const int line = s2 / TR, c0 = 3 * (s2 - line * TR);   // window row (x) or column (y); first slope cell + 1
+      const int step = xs ? 1 : PX;
+      const int first = xs ? (wy0 + line + 2) * PX + wx0 + c0 : (wy0 + c0) * PX + wx0 + line + 2;
+      const int last = Wl + 3 - c0;                   // positions c0 .. Wl + 3 exist
+      const int k3 = 3 < last ? 3 : last, k4 = 4 < last ? 4 : last;
+      const bool two = c0 + 1 < Wl + 2, three = c0 + 2 < Wl + 2;
+      const int os = xs ? 1 : M;                    // next slope cell
+      const int op = xs ? 5 * QXS : 5 * QYS;        // plus states follow the minus states
+      const double* q = sW + v * PY * PX + first;
+      const double q1 = q[step], q2 = q[2 * step], q3 = q[k3 * step];
+      const double d0 = sub(q1, q[0], rk), d1 = sub(q2, q1, rk), d2 = sub(q3, q2, rk);
+      const double d3 = sub(q[k4 * step], q3, rk);
+      const double t0 = mc_half_slope_d(d0, d1, rk), t1 = mc_half_slope_d(d1, d2, rk);
+      const double t2 = mc_half_slope_d(d2, d3, rk);
+      // the base slot lies in the minus half; a partial triple stores no slot past its line
+      double* qm = xs ? sQx + GBH_IX((v * MY + wy0 + line) * (M + 2) + wx0 + c0, 5 * QXS)
+                      : sQy + GBH_IX((v * (MY + 2) + wy0 + c0) * M + wx0 + line, 5 * QYS);
+      qm[0] = sub(q1, t0, rk);
+      qm[op] = add(q1, t0, rk);
+      if (two) {
+        qm[os] = sub(q2, t1, rk);
+        qm[os + op] = add(q2, t1, rk);
+      }
+      if (three) {
+        qm[2 * os] = sub(q3, t2, rk);
+        qm[2 * os + op] = add(q3, t2, rk);
+      }
+    };
+    if constexpr (WIDE) {
+      for (int s = tid; s < (NSX + NSY) * 5; s += NT) slopes(s % (NSX + NSY), s / (NSX + NSY));
+    }
+    for (int s = rtid; !WIDE && s < NSX + NSY + (bf ? 2 : 1) * (Wy + Wx); s += NT) {
       if (bf && s >= NSX + NSY) {
         // the block's boundary faces from the pre-pass: x faces 0 and N of
         // each row, y faces 0 and N of each column (plane k)
@@ -406,39 +470,8 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
         o[0] = F[0]; o[vn * fs] = F[1]; o[vt * fs] = F[2]; o[3 * fs] = F[3]; o[4 * fs] = F[4];
         continue;
       }
-      const bool xs = s < NSX;
-      const int s2 = xs ? s : s - NSX;
-      const int TR = xs ? TRX : TRY, Wl = xs ? Wx : Wy;
-      const int line = s2 / TR, c0 = 3 * (s2 - line * TR);   // window row (x) or column (y); first slope cell + 1
-      const int step = xs ? 1 : PX;
-      const int first = xs ? (wy0 + line + 2) * PX + wx0 + c0 : (wy0 + c0) * PX + wx0 + line + 2;
-      const int last = Wl + 3 - c0;                   // positions c0 .. Wl + 3 exist
-      const int k3 = 3 < last ? 3 : last, k4 = 4 < last ? 4 : last;
-      const bool two = c0 + 1 < Wl + 2, three = c0 + 2 < Wl + 2;
 #pragma unroll 1
-      for (int v = 0; v < 5; ++v) {
-        const int os = xs ? 1 : M;                    // next slope cell
-        const int op = xs ? 5 * QXS : 5 * QYS;        // plus states follow the minus states
-        const double* q = sW + v * PY * PX + first;
-        const double q1 = q[step], q2 = q[2 * step], q3 = q[k3 * step];
-        const double d0 = sub(q1, q[0], rk), d1 = sub(q2, q1, rk), d2 = sub(q3, q2, rk);
-        const double d3 = sub(q[k4 * step], q3, rk);
-        const double t0 = mc_half_slope_d(d0, d1, rk), t1 = mc_half_slope_d(d1, d2, rk);
-        const double t2 = mc_half_slope_d(d2, d3, rk);
-        // the base slot lies in the minus half; a partial triple stores no slot past its line
-        double* qm = xs ? sQx + GBH_IX((v * MY + wy0 + line) * (M + 2) + wx0 + c0, 5 * QXS)
-                        : sQy + GBH_IX((v * (MY + 2) + wy0 + c0) * M + wx0 + line, 5 * QYS);
-        qm[0] = sub(q1, t0, rk);
-        qm[op] = add(q1, t0, rk);
-        if (two) {
-          qm[os] = sub(q2, t1, rk);
-          qm[os + op] = add(q2, t1, rk);
-        }
-        if (three) {
-          qm[2 * os] = sub(q3, t2, rk);
-          qm[2 * os + op] = add(q3, t2, rk);
-        }
-      }
+      for (int v = 0; v < 5; ++v) slopes(s, v);
     }
     __syncthreads();
 
@@ -448,8 +481,9 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
     // (in the inner planes of the ring-2 tile: N full lines of M faces, then
     //     the 4 slab lines at positions [2, N + 2), per direction)
     // (with the pre-pass: the N - 1 inner faces of each line only)
-    const int nper = trim ? N * (N + 8) : bf ? (N - 1) * N : Wx * Wy;
-    for (int f = tid; f < 2 * nper; f += NT) {
+    // (wide CTAs: N + 1 faces of each line, one per thread)
+    const int nper = trim ? N * (N + 8) : bf ? (N - 1) * N : WIDE ? MY * (M + 1) : Wx * Wy;
+    for (int f = tid; f < (WIDE ? nper + (MY + 1) * M : 2 * nper); f += NT) {
       const bool xf = f < nper;
       int i, j;                    // band positions
       const double *ql, *qr;       // minus/plus state arrays, var stride vs
@@ -467,6 +501,7 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
       if (xf) {
         if (trim) { i = pos; j = line; }
         else if (bf) { i = f % (N - 1) + 1; j = f / (N - 1); }
+        else if (WIDE) { i = f % (M + 1); j = f / (M + 1); }
         else { i = f % Wx + wx0; j = f / Wx + wy0; }
         vs = QXS;
         ol = 5 * vs + j * (M + 2) + i;        // plus state of cell i-1 (slot i)
@@ -476,6 +511,7 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
         const int f2 = f - nper;
         if (trim) { i = line; j = pos; }
         else if (bf) { i = f2 % N; j = f2 / N + 1; }
+        else if (WIDE) { i = f2 % M; j = f2 / M; }
         else { i = f2 % Wx + wx0; j = f2 / Wx + wy0; }
         vs = QYS;
         ol = 5 * vs + j * M + i;              // plus state of cell j-1 (slot j)
@@ -503,7 +539,7 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
         (long long)b * L.bstride + ((long long)(k + L.gz) * L.nyp + (cj + L.g)) * L.nxp + (ci + L.g);
     // in an outer plane of a ring stage only the window's cells are updated
     // (the others are never read again and their fluxes were not formed)
-    const bool upd = !outer || (tx >= wx0 && tx < wx1 && ty >= wy0 && ty < wy1);
+    const bool upd = col && (!outer || (tx >= wx0 && tx < wx1 && ty >= wy0 && ty < wy1));
     double out[5];
     const double dtx = reg_const(s_dt[0], zt), dty = reg_const(s_dt[1], zt), dtz = reg_const(s_dt[2], zt);
 #pragma unroll
@@ -519,7 +555,7 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
                : a.combine ? fma(reg_const(a.a, zt), a.Un[o], mul(reg_const(a.b, zt), r, rk)) : r;
       a.Uout[o] = out[v];
     }
-    if (a.flux_slot && col_in && (E == 0 || (k >= 0 && k < L.nz))) {
+    if (a.flux_slot && col && col_in && (E == 0 || (k >= 0 && k < L.nz))) {
       // fluxBuff: fluxes through the block's faces on a coarse-fine boundary,
       // for the correction (interior cells next to the face write them)
       const long long n2 = DIM3 ? N : 1;
@@ -543,7 +579,7 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
       if (DIM3 && k == L.nz - 1 && fsl[FACE_ZP] >= 0)
         for (int v = 0; v < 5; ++v) a.flux_reg[GBH_IX(fsl[FACE_ZP] * ss + (v * n2 + cj) * N + ci, a.flux_reg_len)] = Fzp[v];
     }
-    if (E == 0 && (a.smax_acc || a.Wout)) {
+    if (E == 0 && col && (a.smax_acc || a.Wout)) {
       // calcEos of the new state: the CFL speed, and the next stage's primitives
       double W[5];
       Wide ir;
@@ -560,7 +596,7 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
       }
     }
 
-    if (DIM3) {
+    if (DIM3 && col) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         W0[v] = Wp1[v];
@@ -662,9 +698,10 @@ constexpr int min_ctas() {
 // Work list: items (block, z-chunk, band) in order; each CTA processes
 // `items_per_cta` consecutive items (1 = one CTA per item; a machine-sized
 // grid makes the kernel persistent).  No CTA waits on another.
-template <int N, bool DIM3, int E, int S, bool BF = false>
-__global__ void __launch_bounds__(stage_threads<N, E, S>(), min_ctas<N, E, S>()) stage_kernel(const StageArgs a) {
-  constexpr int NT = stage_threads<N, E, S>();
+template <int N, bool DIM3, int E, int S, bool BF = false, bool WIDE = false>
+__global__ void __launch_bounds__(cta_threads<N, E, S, WIDE>(), WIDE ? 1 : min_ctas<N, E, S>())
+    stage_kernel(const StageArgs a) {
+  constexpr int NT = cta_threads<N, E, S, WIDE>();
   extern __shared__ double smem[];
   __shared__ double s_red[E == 0 && NT > 32 ? NT / 32 : 1];
   __shared__ double s_dt[4];
@@ -672,7 +709,7 @@ __global__ void __launch_bounds__(stage_threads<N, E, S>(), min_ctas<N, E, S>())
   const int first = blockIdx.x * a.items_per_cta;
   const int last = min(nitems, first + a.items_per_cta);
   for (int item = first; item < last; ++item) {
-    stage_item<N, DIM3, E, S, BF>(a, item, smem, s_red, s_dt);
+    stage_item<N, DIM3, E, S, BF, WIDE>(a, item, smem, s_red, s_dt);
     __syncthreads();
   }
 }
@@ -685,18 +722,18 @@ constexpr size_t smem_for() {
                            5 * MY * (M + 1) + 5 * (MY + 1) * M);
 }
 
-template <int N, bool D3, int E, int S, bool BF = false>
+template <int N, bool D3, int E, int S, bool BF = false, bool WIDE = false>
 cudaError_t launch_t(const StageArgs& a, cudaStream_t s) {
   const long long nitems = (long long)(a.block_list ? a.nlist : a.lay.nblocks) * a.nchunks * S;
   const int per = a.items_per_cta > 0 ? a.items_per_cta : 1;
   const unsigned grid = (unsigned)((nitems + per - 1) / per);
-  stage_kernel<N, D3, E, S, BF><<<grid, stage_threads<N, E, S>(), smem_for<N, E, S>(), s>>>(a);
+  stage_kernel<N, D3, E, S, BF, WIDE><<<grid, cta_threads<N, E, S, WIDE>(), smem_for<N, E, S>(), s>>>(a);
   return cudaGetLastError();
 }
 
-template <int N, bool D3, int E, int S, bool BF = false>
+template <int N, bool D3, int E, int S, bool BF = false, bool WIDE = false>
 cudaError_t prepare_one() {
-  return cudaFuncSetAttribute(stage_kernel<N, D3, E, S, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(stage_kernel<N, D3, E, S, BF, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)smem_for<N, E, S>());
 }
 
@@ -705,6 +742,7 @@ template <int N, bool D3>
 cudaError_t prepare_t() {
   cudaError_t e = prepare_one<N, D3, 0, 1>();
   if (e == cudaSuccess) e = prepare_one<N, D3, 0, 1, true>();
+  if (e == cudaSuccess) e = prepare_one<N, D3, 0, wide_bands<N>(), false, true>();
   if (e == cudaSuccess) e = prepare_one<N, D3, 2, 1>();
   if (e == cudaSuccess) e = prepare_one<N, D3, 4, 1>();
   if constexpr (N >= 8) {
@@ -718,7 +756,12 @@ cudaError_t prepare_t() {
 template <int N, bool D3, int E>
 cudaError_t launch_s(const StageArgs& a, cudaStream_t s) {
   if constexpr (N >= 8) {
-    if (a.ysplit == 2) return launch_t<N, D3, E, 2>(a, s);
+    if (a.ysplit == 2 && !a.wide) return launch_t<N, D3, E, 2>(a, s);
+  }
+  if constexpr (E == 0) {
+    if (a.wide)
+      return a.ysplit == wide_bands<N>() && !a.bflux ? launch_t<N, D3, 0, wide_bands<N>(), false, true>(a, s)
+                                                     : cudaErrorInvalidValue;
   }
   if (a.ysplit != 1) return cudaErrorInvalidValue;
   if constexpr (E == 0) {
