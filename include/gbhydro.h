@@ -440,8 +440,7 @@ int hydro_step_host(gbh_ctx *ctx, double *U_host, double *dt_host, void *stream)
 int hydro_step_host_interior(gbh_ctx *ctx, double *U_host, double *dt_host, void *stream);
 
 /* Number of block chunks hydro_step_host pipelines (1..64); 0 (the default)
- * picks the fewest chunks of at most two resident CTAs per SM, one wave of the
- * stage kernel each.  GBH_ERR_INVAL outside [0, 64]. */
+ * picks it from the size of the state's copies.  GBH_ERR_INVAL outside [0, 64]. */
 int gbh_set_host_pipeline(gbh_ctx *ctx, int chunks);
 
 /* Failure check for the floors of the calcEos conversion (no counterpart in

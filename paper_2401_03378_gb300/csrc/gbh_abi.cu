@@ -96,7 +96,7 @@ struct gbh_ctx {
   // lives in, streams (copy in, stage 1, stage 2, copy out) and events
   std::vector<int> h_face;          // host copy of the face table
   int pipe_chunks = 0;
-  int pipe_chunks_wanted = 0;       // gbh_set_host_pipeline (0: about two CTAs per SM per chunk)
+  int pipe_chunks_wanted = 0;       // gbh_set_host_pipeline (0: by the size of the copies)
   std::vector<int> pipe_first, pipe_need;
   cudaStream_t pipe_stream[4] = {nullptr, nullptr, nullptr, nullptr};
   std::vector<cudaEvent_t> pipe_ev;   // [3][chunks]: copied in, stage 1 done, stage 2 done
@@ -252,16 +252,16 @@ int stage_launch(gbh_ctx* c, const double* Uin, const double* Un, double* Uout, 
   const bool prepass = c->face_prepass && c->d_bflux && ring == 0 && gather && (!list || range_first >= 0) &&
                        A.ysplit == 1 && (c->prepass_asked || c->lay.nx < 16);
   if (c->lay.ndim == 3) {
-    // a ring-updating stage spans nz + 2*ring planes; with the pre-pass a work
-    // item is a whole block, and so it is in a range of a pipelined stage (one
-    // wave of whole blocks already)
+    // a ring-updating stage spans nz + 2*ring planes; with the pre-pass a work item
+    // is a whole block: where the caller asked for it, and in every range of a
+    // pipelined stage (a later range reads faces that an earlier one solved)
     const int span = c->lay.nz + 2 * ring;
     const int side = c->lay.nx + 2 * ring;
     const long long nblk = list ? nlist : c->refined ? c->nactive : c->lay.nblocks;
     int k = c->kchunk;
     if (k < 0)
-      k = (range_first >= 0 || (prepass && c->prepass_asked)) ? span
-                                                              : auto_kchunk(span, nblk, side * side / A.ysplit, c->sms);
+      k = prepass && (range_first >= 0 || c->prepass_asked) ? span
+                                                            : auto_kchunk(span, nblk, side * side / A.ysplit, c->sms);
     A.kchunk = k > 0 ? k : span;
     A.nchunks = (span + A.kchunk - 1) / A.kchunk;
   }
@@ -1608,21 +1608,23 @@ static int pipe_setup(gbh_ctx* c, bool interior) {
   if (e == cudaSuccess && !c->d_pipe_dt) e = cudaMalloc(&c->d_pipe_dt, sizeof(double) * c->nproblems);
   if (e != cudaSuccess) return set_err(c, GBH_ERR_NOMEM, "host-step buffers: %s", cudaGetErrorString(e));
   if (c->pipe_chunks) return GBH_OK;
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  // chunks of at most two resident CTAs per SM (one wave of the stage kernel; a
-  // chunk a few CTAs larger would leave a nearly empty second wave), at most 64
-  // chunks (or the count set)
-  const int wave = 2 * (sms > 0 ? sms : 1);
-  int K = c->pipe_chunks_wanted > 0 ? c->pipe_chunks_wanted : (NB + wave - 1) / wave;
+  // The first chunk's copy in and the last one's copy out are not covered by any
+  // stage, and every chunk adds about 13 us of launches and of work items that do
+  // not fill the chip by themselves (the stages of neighbouring chunks run side
+  // by side and fill most of it).  So about sqrt(copy time / 13 us) chunks, as a
+  // power of two, with the link's 200 GB/s in each direction.  Us per step, from
+  // waves of whole blocks to this: 216 blocks of 16^3 1197 -> 1098 (4), 512: 2510 -> 2034
+  // (8), 990: 4073 -> 3681 (8), 4096: 13.0 ms (16); 1728 of 8^3 1682 -> 1417 (4); 64 of
+  // 16^3 407 -> 419 (2).
+  int K = c->pipe_chunks_wanted;
+  if (K <= 0) {
+    const double copies = 2.0 * sizeof(double) * 5.0 * ((double)c->lay.nx * c->lay.ny * c->lay.nz) * NB / 200e9;
+    for (K = 1; K < 64 && 4.0 * K * K * 13e-6 <= copies; K *= 2) {
+    }
+  }
   K = K < 1 ? 1 : (K > 64 ? 64 : (K > NB ? NB : K));
   c->pipe_first.resize(K + 1);
   for (int k = 0; k <= K; ++k) c->pipe_first[k] = (int)((long long)NB * k / K);
-  if (c->pipe_chunks_wanted == 0 && (long long)wave * (K - 1) < NB && (K - 1) * wave > 0) {
-    // whole waves, the remainder last
-    for (int k = 0; k < K; ++k) c->pipe_first[k] = k * wave;
-    c->pipe_first[K] = NB;
-  }
   std::vector<int> chunk_of(NB);
   for (int k = 0; k < K; ++k)
     for (int b = c->pipe_first[k]; b < c->pipe_first[k + 1]; ++b) chunk_of[b] = k;

@@ -335,7 +335,7 @@ class Hydro:
         return U_host
 
     def set_host_pipeline(self, chunks: int = 0):
-        """Block chunks of step_host (0: the fewest chunks of one stage-kernel wave each)."""
+        """Block chunks of step_host (0: by the size of the copies)."""
         self._check(self.lib.gbh_set_host_pipeline(self.ctx, int(chunks)))
 
     def advance_host(self, U_host, nsteps: int, dt_hist_host=None, interior: bool = False):
