@@ -96,6 +96,22 @@ constexpr int wide_threads() {
   return (N / S * (N + 1) + (N / S + 1) * N + 31) / 32 * 32;
 }
 
+// Whether the fluxes of a plane lie over its primitives in shared memory: the
+// primitives are read by the slope list (B) only, so with the boundary fluxes that
+// (B) forms kept in registers until its barrier and one more barrier after the
+// update, an unsplit tile of blocks of 16 takes 68 KB (ring 2: 104 KB) instead of
+// 84 (127), and three (two) CTAs of it fit on an SM instead of two (one).  24 warps
+// of 80 registers against 16 (12) of 128 (157): the FP64 and integer phases of a CTA
+// have more of another's to run beside, which outweighs 500 bytes of spill.
+// 256^3 step 11.59 -> 11.29 ms, 128^3 1.621 -> 1.563 ms, 96-problem 2-D ensemble 4.73 ->
+// 4.39 ms, telescoping 96^3 1.118 -> 1.002 ms.  (Blocks of 8 the same way, 11 CTAs of
+// 64 threads: 105 blocks with three stages 548 -> 576 us, not taken.)
+template <int N, int E, int S, bool WIDE>
+constexpr bool fluxes_over_prims() { return N == 16 && (E == 0 || E == 2) && S == 1 && !WIDE; }
+
+template <int E>
+constexpr int over_prims_ctas() { return E == 0 ? 3 : 2; }
+
 // Row bands of a wide launch.
 template <int N>
 constexpr int wide_bands() { return N == 16 ? 2 : 1; }
@@ -129,10 +145,12 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
   constexpr int QYS = (MY + 2) * M;         // y face states
   constexpr int FXS = MY * (M + 1);         // x fluxes per variable
   constexpr int FYS = (MY + 1) * M;         // y fluxes per variable
+  constexpr bool alias = fluxes_over_prims<N, E, S, WIDE>();
+  constexpr int HEAD = alias ? (5 * PY * PX > 5 * FXS + 5 * FYS ? 5 * PY * PX : 5 * FXS + 5 * FYS) : 5 * PY * PX;
   double* sW = smem;                        // [5][PY][PX] primitives of the band
-  double* sQx = sW + 5 * PY * PX;           // [2][5][MY][M+2] x face states (minus, plus)
+  double* sQx = sW + HEAD;                  // [2][5][MY][M+2] x face states (minus, plus)
   double* sQy = sQx + 2 * 5 * QXS;          // [2][5][MY+2][M] y face states
-  double* sFx = sQy + 2 * 5 * QYS;          // [5][MY][M+1] x fluxes
+  double* sFx = alias ? sW : sQy + 2 * 5 * QYS;   // [5][MY][M+1] x fluxes
   double* sFy = sFx + 5 * FXS;              // [5][MY+1][M] y fluxes
 
   const Layout& L = a.lay;
@@ -422,14 +440,19 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
         qm[2 * os + op] = add(q3, t2, rk);
       }
     };
+    // alias: this thread's boundary flux (the list gives it one at most), kept
+    // until every read of the primitives it goes over is done
+    double Fb[5];
+    double* ob = nullptr;
+    int obv = 0;
+    (void)Fb; (void)ob; (void)obv;
     if constexpr (WIDE) {
       for (int s = tid; s < (NSX + NSY) * 5; s += NT) slopes(s % (NSX + NSY), s / (NSX + NSY));
     }
-    for (int s = rtid; !WIDE && s < NSX + NSY + (bf ? 2 : 1) * (Wy + Wx); s += NT) {
-      if (bf && s >= NSX + NSY) {
-        // the block's boundary faces from the pre-pass: x faces 0 and N of
-        // each row, y faces 0 and N of each column (plane k)
-        const int f = s - NSX - NSY;
+    auto boundary_from_prepass = [&]() {
+      // the block's boundary faces from the pre-pass: x faces 0 and N of
+      // each row, y faces 0 and N of each column (plane k)
+      for (int f = tid; f < 2 * (Wy + Wx); f += NT) {
         const bool xf = f < 2 * N;
         const int side = (xf ? f : f - 2 * N) / N, line = (xf ? f : f - 2 * N) % N;
         const int face = xf ? FACE_XM + side : FACE_YM + side;
@@ -439,8 +462,10 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
           if (xf) sFx[GBH_IX((v * MY + line) * (M + 1) + side * N, 5 * FXS)] = src[v * NF];
           else sFy[GBH_IX((v * (MY + 1) + side * N) * M + line, 5 * FYS)] = src[v * NF];
         }
-        continue;
       }
+    };
+    if (bf && !alias) boundary_from_prepass();
+    for (int s = rtid; !WIDE && s < NSX + NSY + (bf ? 0 : Wy + Wx); s += NT) {
       if (s >= NSX + NSY) {
         const int f = s - NSX - NSY;
         const bool xf = f < Wy;
@@ -467,13 +492,25 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
         const int fs = xf ? FXS : FYS;
         double* o = xf ? sFx + GBH_IX((wy0 + line) * (M + 1) + pos, FXS)
                        : sFy + GBH_IX(pos * M + wx0 + line, FYS);
-        o[0] = F[0]; o[vn * fs] = F[1]; o[vt * fs] = F[2]; o[3 * fs] = F[3]; o[4 * fs] = F[4];
+        if constexpr (alias) {
+          Fb[0] = F[0]; Fb[1] = xf ? F[1] : F[2]; Fb[2] = xf ? F[2] : F[1]; Fb[3] = F[3]; Fb[4] = F[4];
+          ob = o; obv = fs;
+        } else {
+          o[0] = F[0]; o[vn * fs] = F[1]; o[vt * fs] = F[2]; o[3 * fs] = F[3]; o[4 * fs] = F[4];
+        }
         continue;
       }
 #pragma unroll 1
       for (int v = 0; v < 5; ++v) slopes(s, v);
     }
     __syncthreads();
+    if constexpr (alias) {
+      if (bf) boundary_from_prepass();
+      if (ob) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) ob[v * obv] = Fb[v];
+      }
+    }
 
     // (C) HLLC on the x faces (i - 1/2, i in [wx0, wx1)) and y faces (j - 1/2,
     //     j in [wy0, wy1)) of the window; the faces at wx1 - 1/2 and wy1 - 1/2
@@ -596,6 +633,7 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
       }
     }
 
+    if (alias && k + 1 < k1) __syncthreads();   // the next plane's primitives go over the fluxes
     if (DIM3 && col) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
@@ -699,7 +737,10 @@ constexpr int min_ctas() {
 // `items_per_cta` consecutive items (1 = one CTA per item; a machine-sized
 // grid makes the kernel persistent).  No CTA waits on another.
 template <int N, bool DIM3, int E, int S, bool BF = false, bool WIDE = false>
-__global__ void __launch_bounds__(cta_threads<N, E, S, WIDE>(), WIDE ? 1 : min_ctas<N, E, S>())
+__global__ void __launch_bounds__(cta_threads<N, E, S, WIDE>(),
+                                  WIDE ? 1
+                                  : fluxes_over_prims<N, E, S, WIDE>() ? over_prims_ctas<E>()
+                                                                       : min_ctas<N, E, S>())
     stage_kernel(const StageArgs a) {
   constexpr int NT = cta_threads<N, E, S, WIDE>();
   extern __shared__ double smem[];
@@ -714,12 +755,12 @@ __global__ void __launch_bounds__(cta_threads<N, E, S, WIDE>(), WIDE ? 1 : min_c
   }
 }
 
-template <int N, int E, int S>
+template <int N, int E, int S, bool ALIAS = false>
 constexpr size_t smem_for() {
   constexpr int M = N + 2 * E;
   constexpr int MY = M / S;
-  return sizeof(double) * (5 * (MY + 4) * (M + 4) + 2 * 5 * MY * (M + 2) + 2 * 5 * (MY + 2) * M +
-                           5 * MY * (M + 1) + 5 * (MY + 1) * M);
+  constexpr int W = 5 * (MY + 4) * (M + 4), F = 5 * MY * (M + 1) + 5 * (MY + 1) * M;
+  return sizeof(double) * (2 * 5 * MY * (M + 2) + 2 * 5 * (MY + 2) * M + (ALIAS ? (W > F ? W : F) : W + F));
 }
 
 template <int N, bool D3, int E, int S, bool BF = false, bool WIDE = false>
@@ -727,14 +768,15 @@ cudaError_t launch_t(const StageArgs& a, cudaStream_t s) {
   const long long nitems = (long long)(a.block_list ? a.nlist : a.lay.nblocks) * a.nchunks * S;
   const int per = a.items_per_cta > 0 ? a.items_per_cta : 1;
   const unsigned grid = (unsigned)((nitems + per - 1) / per);
-  stage_kernel<N, D3, E, S, BF, WIDE><<<grid, cta_threads<N, E, S, WIDE>(), smem_for<N, E, S>(), s>>>(a);
+  constexpr size_t smem = smem_for<N, E, S, fluxes_over_prims<N, E, S, WIDE>()>();
+  stage_kernel<N, D3, E, S, BF, WIDE><<<grid, cta_threads<N, E, S, WIDE>(), smem, s>>>(a);
   return cudaGetLastError();
 }
 
 template <int N, bool D3, int E, int S, bool BF = false, bool WIDE = false>
 cudaError_t prepare_one() {
   return cudaFuncSetAttribute(stage_kernel<N, D3, E, S, BF, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem_for<N, E, S>());
+                              (int)smem_for<N, E, S, fluxes_over_prims<N, E, S, WIDE>()>());
 }
 
 // The row-band split (S = 2) exists for N >= 8 (a band of at least 4 rows).
