@@ -46,9 +46,9 @@ struct FillMap {
 // region's flags say so.  Every source is an interior cell, so the in-place fill
 // has no read/write overlap.  An offset with no neighbour and no outflow face is
 // left untouched.  512 blocks of 16^3 + 4 guards (199 MB written, 84 MB read, each
-// about 2.4 times, through L2): 136 -> 83 us, bound by the L2 traffic of 32-byte x
+// about 2.4 times, through L2): 136 -> 76 us (83 with 8-byte accesses), bound by the L2 traffic of 32-byte x
 // guards; resolving every cell with 64-bit divisions and table reads was the rest.
-template <bool FAST>
+template <bool FAST, int X>
 __global__ void __launch_bounds__(kThreads) fill_kernel(const FillArgs a, const FillMap m) {
   const Layout& L = a.lay;
   const bool d3 = L.ndim == 3;
@@ -76,7 +76,8 @@ __global__ void __launch_bounds__(kThreads) fill_kernel(const FillArgs a, const 
   __syncthreads();
   const long long lim = (long long)L.nblocks * L.bstride - 4 * L.vstride;
   const unsigned full = 2u * L.g * L.nxp;
-  for (unsigned q = part * kThreads + threadIdx.x; q < m.cells; q += m.parts * kThreads) {
+  for (unsigned t = part * kThreads + threadIdx.x; t < m.cells / X; t += m.parts * kThreads) {
+    const unsigned q = X * t;
     int ii, jj, kk;
     if (q < m.nzg) {
       const unsigned p = div_by<FAST>(q, m.plane), r = q - p * m.plane.d;
@@ -107,11 +108,24 @@ __global__ void __launch_bounds__(kThreads) fill_kernel(const FillArgs a, const 
     const int sk = flags & 4 ? (oz ? L.gz + L.nz - 1 : L.gz) : kk;
     const long long so = GBH_IX(s_shift[e] + (sk * L.nyp + sj) * L.nxp + si, lim);
     const long long dof = GBH_IX((long long)b * L.bstride + (kk * L.nyp + jj) * L.nxp + ii, lim);
-    double v[5];
+    if constexpr (X == 2) {
+      double2 v[5];
+      if (flags & 1) {
 #pragma unroll
-    for (int n = 0; n < 5; ++n) v[n] = a.U[so + n * L.vstride];
+        for (int n = 0; n < 5; ++n) v[n].x = v[n].y = a.U[so + n * L.vstride];
+      } else {
 #pragma unroll
-    for (int n = 0; n < 5; ++n) a.U[dof + n * L.vstride] = v[n];
+        for (int n = 0; n < 5; ++n) v[n] = *reinterpret_cast<const double2*>(a.U + so + n * L.vstride);
+      }
+#pragma unroll
+      for (int n = 0; n < 5; ++n) *reinterpret_cast<double2*>(a.U + dof + n * L.vstride) = v[n];
+    } else {
+      double v[5];
+#pragma unroll
+      for (int n = 0; n < 5; ++n) v[n] = a.U[so + n * L.vstride];
+#pragma unroll
+      for (int n = 0; n < 5; ++n) a.U[dof + n * L.vstride] = v[n];
+    }
   }
 }
 
@@ -395,12 +409,21 @@ cudaError_t launch_fill(const FillArgs& a, cudaStream_t s) {
   // multiply-high quotients: exact while the dividend times the divisor stays
   // below 2^32 (all but blocks of very many planes)
   const bool fast = cells * (unsigned long long)(L.nyp * L.nxp) < (1ull << 32);
-  const long long want = (152LL * 16 + L.nblocks - 1) / L.nblocks, most = (long long)(cells + kThreads - 1) / kThreads;
+  // two cells a thread (16-byte accesses) where every run of guard cells starts on
+  // an even cell of a 16-byte aligned state: nx is even, so an even g does
+  const bool pairs = fast && L.g % 2 == 0 && ((uintptr_t)a.U & 15u) == 0;
+  const long long want = (152LL * 16 + L.nblocks - 1) / L.nblocks;
+  const long long most = (long long)(cells / (pairs ? 2 : 1) + kThreads - 1) / kThreads;
   const int parts = (int)(want < 1 ? 1 : want < most ? want : most);
   const FillMap m{div((unsigned)(L.nyp * L.nxp)), div((unsigned)L.nxp), div(ring), div(2u * L.g),
                   (unsigned)nzg, (unsigned)cells, parts};
   const unsigned grid = (unsigned)(L.nblocks * parts);
-  fast ? fill_kernel<true><<<grid, kThreads, 0, s>>>(a, m) : fill_kernel<false><<<grid, kThreads, 0, s>>>(a, m);
+  if (!fast)
+    fill_kernel<false, 1><<<grid, kThreads, 0, s>>>(a, m);
+  else if (pairs)
+    fill_kernel<true, 2><<<grid, kThreads, 0, s>>>(a, m);
+  else
+    fill_kernel<true, 1><<<grid, kThreads, 0, s>>>(a, m);
   return cudaGetLastError();
 }
 
@@ -422,11 +445,13 @@ cudaError_t launch_dt_reduce(const DtArgs& a, const int* problem, cudaStream_t s
   const Layout& L = a.lay;
   const long long nb = a.block_list ? a.nlist : L.nblocks, per = (long long)L.nx * L.ny * L.nz;
   const int lg = L.nx == 16 ? 4 : L.nx == 8 ? 3 : 2;
-  // shares of a block: enough CTAs to fill the chip, whole rounds of threads each
-  const long long want = (152LL * 8 + nb - 1) / nb, most = (per + kThreads - 1) / kThreads;
-  const int parts = (int)(want < most ? want : most);
-  const long long items = nb * parts;
-  dt_reduce_kernel<<<(int)(items < 152LL * 8 ? items : 152LL * 8), kThreads, 0, s>>>(a, problem, parts, lg);
+  // shares of a block: a power of two (whole rounds of threads), enough CTAs for the
+  // chip's dispatch to even out
+  const long long most = (per + kThreads - 1) / kThreads;
+  int parts = 1;
+  while (parts < most && nb * parts < 152LL * 16) parts *= 2;
+  const long long items = nb * parts, cap = 152LL * 64;
+  dt_reduce_kernel<<<(int)(items < cap ? items : cap), kThreads, 0, s>>>(a, problem, parts, lg);
   return cudaGetLastError();
 }
 
