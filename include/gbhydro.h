@@ -491,7 +491,7 @@ int gbh_fp64_probe(int blocks, int threads, int iters, int lanes, int form, doub
 int gbh_op_count_probe(int fn, int blocks, int threads, int iters, double *io_dev, void *stream);
 
 /* Self-test of the FP64 reciprocal / reciprocal-square-root / square-root
- * building blocks the kernels use (hardware seed + one refinement step):
+ * building blocks the kernels use (integer-pipe forms from an FP32 seed):
  * for n positive, normal, finite DEVICE doubles x_dev writes 6*n DEVICE
  * doubles out_dev = [refined 1/x | IEEE 1/x | refined 1/sqrt(x) |
  * IEEE 1/sqrt(x) | refined sqrt(x) | IEEE sqrt(x)].  Not part of the method. */

@@ -8,11 +8,12 @@
 // primitive variables, and the HLLC flux (Toro's star state, Einfeldt /
 // Roe-average wave-speed bounds).
 //
-// The formulas are arranged to minimise FP64 instructions (the kernel is
-// bound by the FP64 pipe): one reciprocal per primitive conversion, one
-// reciprocal square root per face side giving both sqrt(rho) and 1/rho, the
-// HLLC star state reduced to a single reciprocal, and every comparison done
-// on bit patterns (gbh_fastmath.cuh).  Results agree with the plain
+// The formulas are arranged to keep work off the FP64 pipe, whose warp
+// instruction takes 64 cycles of an SM sub-partition: products, quotients and
+// roots of the equation of state and of the HLLC flux run on the integer pipes in
+// unpacked form (gbh_intmath.cuh), the HLLC star state is reduced to two quotients,
+// every comparison is done on bit patterns (gbh_fastmath.cuh), and what stays FP64
+// are sums and differences of numbers of either sign.  Results agree with the plain
 // formulas to rounding.
 #pragma once
 

@@ -1,7 +1,8 @@
 // gbh_fastmath.cuh -- FP64 building blocks that keep work off the FP64 pipe.
 //
 // On GB300 the FP64 pipe retires 2 lanes per SM per clock while the integer
-// and FP32 pipes retire 64-128; the stage kernel is bound by FP64 issue.  So:
+// and FP32 pipes retire 64-128; with everything in FP64 the stage kernel was bound
+// by FP64 issue at an eighth of the SM's issue slots.  So:
 //  * reciprocal and square root are computed on the integer pipes
 //    (gbh_intmath.cuh), within 0.52 and 0.56 ulp.  They took 3 and 5 FP64
 //    instructions of 64 issue cycles each; 29 of the 80 a face needs.  3-D step

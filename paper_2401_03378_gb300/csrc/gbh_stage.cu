@@ -21,7 +21,8 @@
 //    boundaries, which form their own face states), then the remaining N*N x
 //    faces and N*N y faces are processed as flat work lists over all threads
 //    (full warps, two passes of the CTA for the faces);
-//  - all FP64 arithmetic is register FMAs (gbh_fastmath.cuh);
+//  - products, quotients and roots are integer work (gbh_intmath.cuh); the FP64
+//    arithmetic left is register FMAs (gbh_fastmath.cuh);
 //  - the update of the plane reads its x/y fluxes from shared memory and its
 //    z fluxes from registers and writes Uout.
 // Optional epilogue: calcEos of Uout (the conversion to primitive variables),
