@@ -188,8 +188,8 @@ int auto_kchunk(int span, long long nblk, int threads, int sms) {
   const double w = threads > 32 ? threads / 32.0 : 1.0;
   int best = span;
   double best_t = 1e300;
-  for (int n = 1; n <= span; ++n) {
-    const int k = (span + n - 1) / n;
+  // every chunk length that some number of chunks gives, longest first
+  for (int k = span; k >= 1;) {
     const long long items = nblk * ((span + k - 1) / k);
     const double m = (double)((items + sms - 1) / sms);
     const double t = (k + 0.8) * (w * m > 10.0 ? w * m : 10.0);
@@ -197,6 +197,9 @@ int auto_kchunk(int span, long long nblk, int threads, int sms) {
       best_t = t;
       best = k;
     }
+    if (k == 1) break;
+    const int n = (span + k - 2) / (k - 1);   // the fewest chunks of at most k - 1 planes
+    k = (span + n - 1) / n;
   }
   return best;
 }
