@@ -179,11 +179,11 @@ int record_start(gbh_ctx* c, cudaStream_t s, cudaEvent_t* stop) {
 // of any size takes about as long for a plane as 10 warps' share of a full SM
 // (measured, 16^3 and 8^3 blocks: 18 us a plane alone, 14 us per 8 warps when
 // full).  Against whole blocks, us per step of two stages (in brackets the k
-// chosen here): 8 blocks of 16^3 604 -> 68 (1), 27: 609 -> 143 (1), 125: 641 -> 481
-// (8), 512: 1844 -> 1686 (8), 990: 3251 (16); 105 blocks of 8 x 8 x 12: 408 -> 131
-// (2), 512 of 8^3 360 -> 296 (4), 990: 529 (8); telescoping, 216 blocks of 16^3: 1474
-// -> 1189.  Over the k measured beside it (2, 3, 4, 6, 8 and whole blocks) the choice
-// is the fastest, or within 10% of it.
+// chosen here): 8 blocks of 16^3 638 -> 70 (1), 27: 641 -> 119 (1), 125: 697 -> 497
+// (8), 512: 1842 -> 1565 (8), 990: 3027 (16); 105 blocks of 8 x 8 x 12: 408 -> 131
+// (2), 512 of 8^3 360 -> 296 (4), 990: 529 (8); telescoping, 216 blocks of 16^3: 1293
+// -> 1005.  Over 20 lattices and the k measured beside it (2, 3, 4, 6, 8 and whole
+// blocks) the choice is the fastest or within 8% of it, once (80 blocks) within 15%.
 int auto_kchunk(int span, long long nblk, int threads, int sms) {
   const double w = threads > 32 ? threads / 32.0 : 1.0;
   int best = span;
