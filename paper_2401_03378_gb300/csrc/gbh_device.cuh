@@ -136,9 +136,6 @@ __device__ __forceinline__ double mc_half_slope_d(double dm, double dp, const Rk
   return bitsd((long long)half_slope(word_pair(dm), word_pair(dp)));
 }
 
-// x / 2 for a positive normal x >= 2^-1021 (one off the exponent field)
-__device__ __forceinline__ double half_pos(double x) { return bitsd(dbits(x) - (1LL << 52)); }
-
 // max(a, b) of non-negative doubles on the integer pipe (their bit patterns
 // order like their values; fmax is an FP64-pipe instruction).  A NaN operand
 // is passed over, as fmax passes it over.

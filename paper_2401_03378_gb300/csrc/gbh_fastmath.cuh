@@ -23,9 +23,7 @@
 //    constants (1, -0, the equation-of-state constants, dt/dx) get there
 //    through reg_const: their bit patterns OR-ed with a run-time zero that
 //    depends on the thread index, so the compiler can neither fold them into
-//    constant operands nor keep them in uniform registers.  With the
-//    compile-time constants of plain_rk() the same code compiles to the
-//    ordinary DADD / DMUL.
+//    constant operands nor keep them in uniform registers.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -42,8 +40,6 @@ __device__ __forceinline__ double bitsd(long long b) { return __longlong_as_doub
 __device__ __forceinline__ double add(double a, double b, const Rk& k) { return fma(a, k.one, b); }
 __device__ __forceinline__ double sub(double a, double b, const Rk& k) { return fma(-b, k.one, a); }
 __device__ __forceinline__ double mul(double a, double b, const Rk& k) { return fma(a, b, k.nz); }
-
-__device__ __forceinline__ Rk plain_rk() { return Rk{1.0, -0.0}; }
 
 // A run-time zero that depends on the thread index (p.opaque is 0).
 __device__ __forceinline__ long long thread_zero(const Eos& p) { return p.opaque & (long long)threadIdx.x; }
