@@ -123,7 +123,7 @@ __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double W
   const Wide CL2 = wide_mul(GPL, IL), CR2 = wide_mul(GPR, IR);
   const Wide CL = wide_sqrt(CL2), CR = wide_sqrt(CR2);
   const Wide Q = wide_mul(sP, iP);                           // 1/sqrt(rho_L rho_R)
-  const Wide D = wide_rcp(wide_add(sP, RR));
+  const Wide D = wide_rcp_low(wide_add(sP, RR));
   const Wide XL = wide_mul(sP, D), XR = wide_mul(RR, D);     // Roe weights
   const double q = wide_double(Q), q2 = wide_double(iP);
   const double iL = wide_double(IL), iR = wide_double(IR);

@@ -250,7 +250,7 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
   const Wide cL2 = wide_mul(wide_of(pL), wide_mul(RR, g_P)), cR2 = wide_mul(wide_of(pR), wide_mul(RL, g_P));
   const double cL = wide_double(wide_sqrt(cL2)), cR = wide_double(wide_sqrt(cR2));
   const Wide sP = wide_sqrt(P);
-  const Wide D = wide_rcp(wide_add(sP, RR));
+  const Wide D = wide_rcp_low(wide_add(sP, RR));
   const Wide wl = wide_mul(sP, D), wr = wide_mul(RR, D);   // Roe weights
 
   const double du = sub(uL, uR, k), dv = sub(vL, vR, k), dw = sub(wL, wR, k);

@@ -14,7 +14,8 @@
 // Wide: a positive number as a 63-bit mantissa and an exponent,
 //     value = (h 2^32 + l) 2^(e - 1023 - 62),  2^62 <= h 2^32 + l < 2^63,
 // e in the biased form of a double; a reciprocal, a root or a product of them may
-// be up to 64 units below 2^62, which products, sums, roots and the rounding take.  Products,
+// be up to 64 units below 2^62, which products, sums, roots and the rounding take
+// (and wide_rcp_low, where a reciprocal is taken of one).  Products,
 // reciprocals and roots are computed to a relative error below 2^-58 (stated at
 // each), so a double rounded from a chain of them (wide_pack, to nearest) is
 // within 0.55 ulp of the exact value: tighter than the same chain of FP64
@@ -162,7 +163,7 @@ GBH_HD Wide wide_add(const Wide& a, const Wide& b) {
 }
 
 // 1 / a: relative error below 2^-58.5.  a is at least 2^62: unpacked, a product
-// of unpacked numbers, or a sum with one of them.
+// of unpacked numbers, or a sum whose larger term is one of them.
 GBH_HD Wide wide_rcp(const Wide& a) {
   using namespace imath;
   // seed: R0 = 1/f in units of 2^-31, f in [1, 2) the leading 24 bits of a; n0 = -R0
@@ -184,6 +185,15 @@ GBH_HD Wide wide_rcp(const Wide& a) {
   r.l = ~(lo32(c) << 3);
   r.e = 2045 - a.e;
   return r;
+}
+
+// 1 / a of a number that may lie below 2^62, as a sum whose larger term is a root:
+// taken as 2^62 there, which changes the result by as many units of 2^-62 as it
+// lies below (three for a root).  wide_rcp itself is off by 2^-21 on such numbers:
+// its seed's 1/f exceeds 1.  Three instructions, so not in every reciprocal.
+GBH_HD Wide wide_rcp_low(const Wide& a) {
+  const bool low = a.h < 0x40000000u;
+  return wide_rcp(Wide{low ? 0x40000000u : a.h, low ? 0u : a.l, a.e});
 }
 
 // sqrt(a): relative error below 2^-57.

@@ -1,0 +1,48 @@
+"""Stages and time steps on states at the edges of the accepted range, against
+the oracle or against the plain definition."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as wl
+from oracle.oracle import Oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gb():
+    import paper_2401_03378_gb300 as gb
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return gb
+
+
+def state(lat, rho, u, v, w, p):
+    return np.ascontiguousarray(np.moveaxis(wl.conserved(rho, u, v, w, p, 1.4), 0, 1))
+
+
+@pytest.mark.parametrize("k", [40, 120, 130, 140])
+@pytest.mark.parametrize("u1,u2", [(0.0, 0.0), (0.5, 0.25)])
+def test_a_power_of_two_floor_beside_unit_density(gb, k, u1, u2):
+    """Half the domain at density and pressure 1, the other half at the floors
+    2^-k: one stage, within 1e-13 of each variable's largest value."""
+    lat = wl.lattice_2d(4, 4, 8, 8, 4, bc="periodic")
+    X, Y, _ = wl.cell_centers(lat)
+    q = np.where(X < 0.5, 1.0, 2.0 ** -k)
+    z = np.zeros_like(q)
+    U = state(lat, q, np.where(X < 0.5, u1, u2), z, z, q)
+    kw = dict(small_rho=2.0 ** -k, small_p=2.0 ** -(k + 60))
+    h, o = gb.Hydro.from_lattice(lat, **kw), Oracle(lat, **kw)
+    dt = 0.2 * lat.dx[0]
+    Ud = torch.from_numpy(U.copy()).cuda()
+    out = torch.zeros_like(Ud)
+    h.stage(Ud, None, out, dt, 0.0, 1.0)
+    Uf, ref = U.copy(), np.zeros_like(U)
+    o.fill_guardcells(Uf)
+    o.stage(Uf, U, ref, dt, 0.0, 1.0)
+    zs, ys, xs = lat.interior_slices()
+    got = out.cpu().numpy()
+    for v in range(5):
+        a, b = got[:, v, zs, ys, xs], ref[:, v, zs, ys, xs]
+        assert np.max(np.abs(a - b)) <= 1e-13 * np.max(np.abs(b)), v
