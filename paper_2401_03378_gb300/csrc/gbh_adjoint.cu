@@ -115,23 +115,21 @@ __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double W
   // ---- forward ----
   // From the densities and pressures to the sound speeds and Roe weights, and
   // the quotients S* and t, as in hllc_flux: Wide numbers on the integer pipes.
-  const uint32_t bad = non_finite_mask(WL, WR);
+  uint32_t bad = non_finite_mask(WL, WR);
   const Wide RL = wide_of(rL), RR = wide_of(rR);
   const Wide P = wide_mul(RL, RR), iP = wide_rcp(P), sP = wide_sqrt(P);
-  const Wide GPL = wide_mul(e.wgamma, wide_of(pL)), GPR = wide_mul(e.wgamma, wide_of(pR));
   const Wide IL = wide_mul(RR, iP), IR = wide_mul(RL, iP);   // 1/rho
-  const Wide CL2 = wide_mul(GPL, IL), CR2 = wide_mul(GPR, IR);
+  const Wide CL2 = wide_mul(wide_mul(e.wgamma, wide_of(pL)), IL), CR2 = wide_mul(wide_mul(e.wgamma, wide_of(pR)), IR);
   const Wide CL = wide_sqrt(CL2), CR = wide_sqrt(CR2);
-  const Wide Q = wide_mul(sP, iP);                           // 1/sqrt(rho_L rho_R)
   const Wide D = wide_rcp_low(wide_add(sP, RR));
   const Wide XL = wide_mul(sP, D), XR = wide_mul(RR, D);     // Roe weights
-  const double q = wide_double(Q), q2 = wide_double(iP);
-  const double iL = wide_double(IL), iR = wide_double(IR);
-  const double gpL = wide_double(GPL), gpR = wide_double(GPR);
-  const double cL2 = wide_double(CL2), cR2 = wide_double(CR2);
+  // these can leave the range of a double; a 1/rho that does leaves no gradient
+  const double iL = wide_signed(IL, 0u), iR = wide_signed(IR, 0u);
+  bad |= IL.e < 1 || IR.e < 1 ? 0x7fffffffu : 0u;
+  const double cL2 = wide_signed(CL2, 0u), cR2 = wide_signed(CR2, 0u);
   const double cL = wide_double(CL), cR = wide_double(CR);
   const double qL = wide_double(wide_rcp(wide_of(cL))), qR = wide_double(wide_rcp(wide_of(cR)));   // 1/c
-  const double r = wide_double(wide_mul(RR, Q));             // sqrt(rho_R / rho_L)
+  const double r = wide_double(wide_mul(sP, IL));            // sqrt(rho_R / rho_L)
   const double wl = wide_double(XL), wr = wide_double(XR);
   const double ut = fma(wl, uL, M(wr, uR));
   const double du = S(uL, uR), dv = S(vL, vR), dw = S(wL, wR);
@@ -151,6 +149,7 @@ __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double W
   const Wide RD = wide_rcp(wide_add(ML, MR));              // -1 / (mL - mR)
   const double rd = wide_signed(RD, 0x80000000u);
   const double num = fma(-mR, uR, fma(mL, uL, S(pR, pL)));
+  bad |= overflow_mask(du2, num);
   const Wide WS = wide_mul(wide_of0(num), RD);
   const uint32_t ssgn = sign01(num) ^ 1u;
   const double Ss = wide_signed(WS, ssgn << 31 | bad);
@@ -168,8 +167,8 @@ __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double W
   const double t = sel(fan, wide_signed(wide_mul(WS, DKR), (ssgn ^ dsgn) << 31 | bad), uK);
   const double g = S(t, uK);
   const double kK = fma(wK, wK, fma(vK, vK, M(uK, uK)));
-  const Wide RK = wide_of(rK), KIN = wide_mul(RK, wide_of(kK));
-  const double hK = wide_double(wide_add(Wide{KIN.h, KIN.l, KIN.e - 1}, wide_mul(e.wg_gm1, wide_of(pK))));
+  const Wide RK = wide_of(rK), KIN = wide_mul(RK, wide_of_squares(kK));
+  const double hK = wide_signed(wide_add(Wide{KIN.h, KIN.l, KIN.e - 1}, wide_mul(e.wg_gm1, wide_of(pK))), 0u);
   const double gm = M(g, mK);
   const double F0 = M(rK, t);
   // ---- reverse ----
@@ -271,17 +270,11 @@ __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double W
   // cL2 = gamma pL iL, cR2 = gamma pR iR
   bpL = fma(M(bcL2, iL), e.gamma, bpL);
   bpR = fma(M(bcR2, iR), e.gamma, bpR);
-  const double biL = M(bcL2, gpL), biR = M(bcR2, gpR);
-  // iL = rR q2, iR = rL q2, r = rR q, q2 = q q
-  brR = fma(biL, q2, brR);
-  brL = fma(biR, q2, brL);
-  const double bq2 = fma(biL, rR, M(biR, rL));
-  brR = fma(br, q, brR);
-  const double bq = fma(br, rR, M(A(bq2, bq2), q));
-  // q = (rL rR)^(-1/2): d q / d(rL rR) = -q^3 / 2
-  const double nbP = M(M(half_any(bq), q), q2);
-  brL = fma(-nbP, rR, brL);
-  brR = fma(-nbP, rL, brR);
+  // and d cL2 / d rL = -cL2 / rL, r = sqrt(rR / rL); each term by one 1/rho, so that
+  // no product of two densities or of two reciprocals leaves the range
+  const double hr = M(half_any(br), r);                    // rR times the adjoint through r
+  brL = fma(-fma(bcL2, cL2, hr), iL, brL);
+  brR = fma(S(hr, M(bcR2, cR2)), iR, brR);
   bWL[0] = brL; bWL[1] = buL; bWL[2] = bvL; bWL[3] = bwL; bWL[4] = bpL;
   bWR[0] = brR; bWR[1] = buR; bWR[2] = bvR; bWR[3] = bwR; bWR[4] = bpR;
 }

@@ -45,11 +45,20 @@ __device__ __forceinline__ Wide wide_of0(double x) {
 }
 
 // Wide -> double with the bits of `top` (a sign bit; a NaN's exponent and
-// quiet bits) OR-ed in: below the normal range a zero, above it an infinity or NaN.
+// quiet bits) OR-ed in: below the normal range a zero, above it an infinity.
 __device__ __forceinline__ double wide_signed(const Wide& a, uint32_t top) {
-  const uint64_t m = wide_pack(Wide{a.h, a.l, a.e < 2047 ? a.e : 2047});
-  const bool in = a.e >= 1;
-  return bitsd((long long)imath::pair((in ? imath::hi32(m) : 0u) | top, in ? imath::lo32(m) : 0u));
+  const uint64_t m = wide_pack(a);
+  const bool in = (unsigned)(a.e - 1) < 2046u;
+  const uint32_t out = a.e > 0 ? 0x7ff00000u : 0u;
+  return bitsd((long long)imath::pair((in ? imath::hi32(m) : out) | top, in ? imath::lo32(m) : 0u));
+}
+
+// The unpacked magnitude of a sum of squares, with an infinity as a number so
+// large that no product of the scheme brings it back into the range of a double.
+__device__ __forceinline__ Wide wide_of_squares(double x) {
+  Wide a = wide_of(x);
+  a.e = a.e == 2047 ? 8192 : a.e;
+  return a;
 }
 
 // 0 or 1: the sign of x (as a number, not a masked word: the compiler turns an
@@ -58,6 +67,11 @@ __device__ __forceinline__ uint32_t sign01(double x) { return hi_word(x) >> 31; 
 
 // Infinity or NaN.
 __device__ __forceinline__ bool not_finite(double x) { return (hi_word(x) & 0x7ff00000u) == 0x7ff00000u; }
+
+// A NaN's high word where one of two sums of finite terms overflowed, else 0.
+__device__ __forceinline__ uint32_t overflow_mask(double a, double b) {
+  return not_finite(a) || not_finite(b) ? 0x7fffffffu : 0u;
+}
 
 // See hllc_flux.
 __device__ __forceinline__ uint32_t non_finite_mask(const double WL[5], const double WR[5]) {
@@ -241,7 +255,7 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
   // +0, or a NaN's bits when any input is not finite (FP32 arithmetic on the
   // high words, whose exponent field is all ones for an infinity, a NaN or a
   // magnitude from 2^1017): OR-ed into S* and t, from where it reaches every flux
-  const uint32_t bad = non_finite_mask(WL, WR);
+  uint32_t bad = non_finite_mask(WL, WR);
 
   // the wave speeds' positive part, on the integer pipes
   const Wide RL = wide_of(rL), RR = wide_of(rR);
@@ -255,7 +269,8 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
 
   const double du = sub(uL, uR, k), dv = sub(vL, vR, k), dw = sub(wL, wR, k);
   const double ut = fma(-wide_double(wr), du, uL);         // w_L u_L + w_R u_R
-  const Wide du2 = wide_of(fma(dw, dw, fma(dv, dv, mul(du, du, k))));
+  const double du2_d = fma(dw, dw, fma(dv, dv, mul(du, du, k)));
+  const Wide du2 = wide_of(du2_d);
   const Wide ct2 = wide_add(wide_mul(wl, cL2),
                             wide_mul(wr, wide_add(cR2, wide_mul(wide_mul(e.whgm1, wl), du2))));
   const double ct = wide_double(wide_sqrt(ct2));
@@ -268,6 +283,7 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
   const double mL = wide_signed(ML, 0x80000000u), mR = wide_signed(MR, 0u);
   // S* = num / (m_L - m_R) = -num / (|m_L| + |m_R|)
   const double num = fma(-mR, uR, fma(mL, uL, sub(pR, pL, k)));
+  bad |= overflow_mask(du2_d, num);                        // which the unpacked form would take as 2^1024
   const Wide WS = wide_mul(wide_of0(num), wide_rcp(wide_add(ML, MR)));
   const uint32_t ssgn = sign01(num) ^ 1u;
   const double Ss = wide_signed(WS, ssgn << 31 | bad);
@@ -287,8 +303,8 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
   const double g = sub(t, uK, k);
   const Wide RK = wide_of(rK);
   // E + p of the chosen side
-  const Wide kin = wide_mul(RK, wide_of(fma(wK, wK, fma(vK, vK, mul(uK, uK, k)))));
-  const double hK = wide_double(wide_add(Wide{kin.h, kin.l, kin.e - 1}, wide_mul(e.wg_gm1, wide_of(pK))));
+  const Wide kin = wide_mul(RK, wide_of_squares(fma(wK, wK, fma(vK, vK, mul(uK, uK, k)))));
+  const double hK = wide_signed(wide_add(Wide{kin.h, kin.l, kin.e - 1}, wide_mul(e.wg_gm1, wide_of(pK))), 0u);
   const Wide F0 = wide_mul(RK, T);
   const Wide GM = wide_mul(wide_of0(g), left ? ML : MR);   // |g m_K|
   const uint32_t gmsgn = sign01(g) ^ (left ? 1u : 0u);

@@ -46,3 +46,25 @@ def test_a_power_of_two_floor_beside_unit_density(gb, k, u1, u2):
     for v in range(5):
         a, b = got[:, v, zs, ys, xs], ref[:, v, zs, ys, xs]
         assert np.max(np.abs(a - b)) <= 1e-13 * np.max(np.abs(b)), v
+
+
+@pytest.mark.parametrize("k", [-400, 300, 500, 511, 530, 600, 900])
+def test_scaled_states(gb, k):
+    """The update is homogeneous in (rho, momentum, E): a state times 2^k gives
+    2^k times the result, and the same vector-Jacobian product."""
+    lat = wl.lattice_2d(3, 3, 8, 8, 4, bc="periodic")
+    U0 = wl.random_state(lat, seed=11, rough=False)
+    rng = np.random.default_rng(12)
+    M = torch.from_numpy(rng.normal(size=U0.shape)).cuda()
+    h = gb.Hydro.from_lattice(lat, small_rho=1e-150, small_p=1e-200)
+    zs, ys, xs = lat.interior_slices()
+    res = []
+    for s in (1.0, 2.0 ** k):
+        U = torch.from_numpy(U0 * s).cuda()
+        out, lam = torch.zeros_like(U), torch.zeros_like(U)
+        h.stage(U, None, out, 1e-3, 0.0, 1.0)
+        h.stage_vjp(U, M, 1e-3, out=lam)
+        res.append((out[:, :, zs, ys, xs].cpu().numpy() / s, lam[:, :, zs, ys, xs].cpu().numpy()))
+    (a, la), (b, lb) = res
+    assert np.max(np.abs(a - b)) <= 1e-13 * np.max(np.abs(a))
+    assert np.max(np.abs(la - lb)) <= 1e-12 * np.max(np.abs(la))
