@@ -132,8 +132,9 @@ __global__ void __launch_bounds__(kThreads) fill_kernel(const FillArgs a, const 
 // CFL reduction: max over the interior cells of the signal-speed sum, into
 // smax_acc, or with `problem` into the accumulator of the block's problem (one
 // atomicMax per CTA and block on the bit pattern, which orders like the
-// non-negative value).  A CTA takes one of `parts` shares of the blocks' cells;
-// nx = ny = 2^lg.  512 blocks of 16^3: 92 -> 54 us (the 64-bit divisions of a cell
+// non-negative value).  A CTA takes one of `parts` shares of a block's cells; with
+// parts = 0 the next kThreads cells of the list's blocks one after another (blocks
+// of fewer cells; no `problem`).  nx = ny = 2^lg.  512 blocks of 16^3: 92 -> 54 us (the 64-bit divisions of a cell
 // index and 22 FP64 instructions a cell are gone).
 __global__ void __launch_bounds__(kThreads) dt_reduce_kernel(const DtArgs a, const int* problem, int parts, int lg) {
   const Layout& L = a.lay;
@@ -142,17 +143,29 @@ __global__ void __launch_bounds__(kThreads) dt_reduce_kernel(const DtArgs a, con
   const long long zt = thread_zero(a.eos);
   const Eos e = reg_eos(a.eos, zt);   // FP64 constants in per-thread registers (gbh_fastmath.cuh)
   __shared__ double red[kThreads / 32];
-  const int items = (a.block_list ? a.nlist : L.nblocks) * parts;
+  const int nb = a.block_list ? a.nlist : L.nblocks;
+  const unsigned total = (unsigned)nb * per;          // with parts = 0 (below 2^32: the state would not fit)
+  const int items = parts ? nb * parts : (int)((total + kThreads - 1) / kThreads);
   double smax = 0.0;
   for (int s = blockIdx.x; s < items; s += gridDim.x) {
-    const int slot = s / parts, part = s - slot * parts;
+    int slot, part = 0;
+    unsigned cell = threadIdx.x;
+    if (parts) {
+      slot = s / parts;
+      part = s - slot * parts;
+    } else {
+      const unsigned first = (unsigned)s * kThreads, lo = first / per, t = first - lo * per + threadIdx.x, sub = t / per;
+      slot = (int)(lo + sub);
+      cell = t - sub * per;
+      if (slot >= nb) break;                           // no barrier in this form's loop
+    }
     const int b = a.block_list ? __ldg(a.block_list + slot) : slot;
     const double ix = reg_const(__ldg(a.inv_dx + 3 * b), zt), iy = reg_const(__ldg(a.inv_dx + 3 * b + 1), zt);
     const double iz = reg_const(__ldg(a.inv_dx + 3 * b + 2), zt);
     const double isum = inv_width_sum(e, ix, iy, iz, d3);
     const double* src = a.U + GBH_IX((long long)b * L.bstride, (long long)L.nblocks * L.bstride);
     if (problem) smax = 0.0;
-    for (unsigned t = part * kThreads + threadIdx.x; t < per; t += parts * kThreads) {
+    for (unsigned t = part * kThreads + cell; t < per; t += (parts ? parts : 1) * kThreads) {
       const int i = t & (L.nx - 1), j = (t >> lg) & (L.nx - 1), k = t >> (2 * lg);
       const long long o = GBH_IX(((long long)(k + L.gz) * L.nyp + (j + L.g)) * L.nxp + (i + L.g), L.vstride);
       double U[5], W[5];
@@ -450,7 +463,10 @@ cudaError_t launch_dt_reduce(const DtArgs& a, const int* problem, cudaStream_t s
   const long long most = (per + kThreads - 1) / kThreads;
   int parts = 1;
   while (parts < most && nb * parts < 152LL * 16) parts *= 2;
-  const long long items = nb * parts, cap = 152LL * 64;
+  // blocks smaller than a CTA one after another, where they have no problems of
+  // their own: a CTA with a block of 4^2 to itself has 16 of 256 threads at work
+  if (!problem && per < kThreads) parts = 0;
+  const long long items = parts ? nb * parts : (nb * per + kThreads - 1) / kThreads, cap = 152LL * 64;
   dt_reduce_kernel<<<(int)(items < cap ? items : cap), kThreads, 0, s>>>(a, problem, parts, lg);
   return cudaGetLastError();
 }
