@@ -143,29 +143,43 @@ int gbh_create_refined_batched(const gbh_params *params, const gbh_refinement *r
 
 /* Work decomposition of the stage kernel (how the concurrent-data pattern of
  * Sec. 3.2 maps blocks onto CTAs; not a choice the paper makes): kchunk = z planes per work item
- * (3-D; 0 or nzb = the whole block; a new context picks it per launch from
- * the number of blocks and SMs) and items_per_cta = consecutive work
- * items one CTA processes (1 = a CTA per item; a grid of about two CTAs per
- * SM makes the kernel persistent).  A third choice is the tile: the plane
+ * (3-D; 0 or nzb = the whole block; -1, the default of a new context = picked
+ * per launch from the number of blocks and SMs, with a CTA of a thread per face
+ * where there are few items) and items_per_cta = consecutive work
+ * items one CTA processes (1 = a CTA per item; a grid of as many CTAs as fit on
+ * the SMs makes the kernel persistent).  A third choice is the tile: the plane
  * tile of a work item (the nxb x nyb block plane, widened by the ring in the
  * telescoping mode) can be cut into ysplit row bands, one CTA each, so a CTA
- * has 1/ysplit of the threads and shared memory (twice as many CTAs fit on
+ * has 1/ysplit of the threads and shared memory (more CTAs fit on
  * an SM) at the cost of the halo rows and faces both bands form at the cut;
  * gbh_set_tile_split(ctx, ring, ysplit) sets it per ring width (0: the
  * interior stage; 2, 4: the ring stages of the telescoping mode), ysplit 1,
  * or 2 for blocks of at least 8 cells per side.  Results do not depend on
- * any of these (bitwise).  gbh_autotune times the candidates on U (stage
- * launches into the context's scratch; U is not modified; synchronises the
- * stream; clears the floor counter) and keeps the fastest: kchunk x
- * items_per_cta x ysplit for the interior stage, and, in the telescoping
- * mode, ysplit for each ring stage.  gbh_set_decomposition sets kchunk and
- * items_per_cta directly.  The chosen kchunk and items_per_cta are written to
- * *kchunk_out / *items_out if not NULL; gbh_get_tile_split reads a split.
- * GBH_ERR_INVAL: a ring other than 0, 2, 4 or an unsupported ysplit. */
+ * any of these (bitwise).
+ * gbh_autotune times the default (kchunk -1, one item per CTA, unsplit) and
+ * fixed choices on U (stage launches into the context's scratch; U is not
+ * modified; synchronises the stream; clears the floor counter) and keeps a
+ * fixed choice where it is at least 2% faster, else the default: kchunk x
+ * items_per_cta x ysplit for the interior stage and, in the telescoping
+ * mode, for each ring stage.  The ranges of a pipelined host
+ * step stay as they were.  The kchunk and items_per_cta of the interior stage
+ * are written to *kchunk_out / *items_out if not NULL, the default and whole
+ * blocks as kchunk = nzb; after an error the decomposition is the one before.
+ * gbh_set_decomposition sets kchunk and items_per_cta of every stage,
+ * gbh_get_decomposition reads those of the interior stage (0 for whole blocks,
+ * -1 for the default) and gbh_get_tile_split reads a split.  gbh_stage_plan
+ * writes what a stage of ring width `ring` over all blocks takes with the
+ * context's settings: plan[0] = z planes per work item, [1] = items per CTA,
+ * [2] = row bands, [3] = 1 with a thread per face, [4] = 1 with the face
+ * pre-pass below.
+ * GBH_ERR_INVAL: a ring other than 0, 2, 4, an unsupported ysplit, or a kchunk
+ * outside [-1, nzb] (2-D: other than -1 and 0). */
 int gbh_autotune(gbh_ctx *ctx, const double *U, int *kchunk_out, int *items_out, void *stream);
 int gbh_set_decomposition(gbh_ctx *ctx, int kchunk, int items_per_cta);
+int gbh_get_decomposition(gbh_ctx *ctx, int *kchunk, int *items_per_cta);
 int gbh_set_tile_split(gbh_ctx *ctx, int ring, int ysplit);
 int gbh_get_tile_split(gbh_ctx *ctx, int ring, int *ysplit);
+int gbh_stage_plan(gbh_ctx *ctx, int ring, int plan[5]);
 
 /* Time-stepping mode (Sec. 4.2, the telescoping variant of the SSP-RK
  * stepper).  enable = 0 (the default): non-telescoping, the guard cells are

@@ -22,6 +22,13 @@
 using gbh::Eos;
 using gbh::Layout;
 
+// Work decomposition of a stage launch.
+struct Decomp {
+  int kchunk = -1;          // z planes per work item (3-D); 0 = the whole block, -1 = by auto_kchunk
+  int items_per_cta = 1;
+  int ysplit = 1;           // row bands of the plane tile
+};
+
 struct gbh_ctx {
   Layout lay{};
   Eos eos{};
@@ -70,11 +77,11 @@ struct gbh_ctx {
   int* d_problem = nullptr;
   unsigned long long* d_smax = nullptr;  // [nproblems]; points into d_words for a single problem
   unsigned long long* d_smax_own = nullptr;
-  // stage-kernel work decomposition (gbh_autotune)
-  int kchunk = -1;                  // z planes per work item (3-D); 0 = the whole block, -1 = by auto_kchunk
+  // stage-kernel work decomposition (gbh_set_decomposition, gbh_set_tile_split,
+  // gbh_autotune): stages of ring width 0, 2 and 4, and a block range of a
+  // pipelined stage (hydro_step_host), which the autotuner does not time
+  Decomp dec[3], dec_range;
   int sms = 0;                      // SMs of the device
-  int items_per_cta = 1;
-  int ysplit[3] = {1, 1, 1};        // row bands of the plane tile for ring widths 0, 2, 4
   // CUDA graph of hydro_advance_graph
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t graph_exec = nullptr;
@@ -220,6 +227,43 @@ bool take_wide(int nx, bool dim3, long long items, int sms) {
   return !dim3 || items <= 2LL * sms;
 }
 
+// What a stage launch over nblk blocks takes (0: all the blocks it would update);
+// listed: over a block list of the caller's, ranged: one of a sequence of block
+// ranges (see stage_launch).
+struct StagePlan {
+  int kchunk, nchunks, items_per_cta, ysplit;
+  bool wide, prepass;
+};
+
+StagePlan plan_stage(const gbh_ctx* c, int ring, bool gather, long long nblk, bool listed, bool ranged) {
+  const Layout& L = c->lay;
+  const Decomp d = ranged ? c->dec_range : ring == 0 || ring == 2 || ring == 4 ? c->dec[ring / 2] : Decomp{};
+  if (nblk <= 0) nblk = c->refined ? c->nactive : L.nblocks;
+  StagePlan p{1, 1, d.items_per_cta, d.ysplit, false, false};
+  // The face pre-pass by default only below 16 cells per side: a block of 16^3
+  // has few boundary faces for what the extra launch and its buffer cost now
+  // that a face takes 19 FP64 instructions (4096 blocks of 16^3: 12.32 ms a step
+  // with it, 12.17 without; 4096 blocks of 8^3: 1.86 and 2.09).
+  p.prepass = c->face_prepass && c->d_bflux && ring == 0 && gather && (!listed || ranged) && p.ysplit == 1 &&
+              (c->prepass_asked || L.nx < 16);
+  if (L.ndim == 3) {
+    // a ring-updating stage spans nz + 2*ring planes; with the pre-pass a work item
+    // is a whole block: where the caller asked for it, and in every range of a
+    // pipelined stage (a later range reads faces that an earlier one solved)
+    const int span = L.nz + 2 * ring, side = L.nx + 2 * ring;
+    int k = d.kchunk;
+    if (k < 0) k = p.prepass && (ranged || c->prepass_asked) ? span : auto_kchunk(span, nblk, side * side / p.ysplit, c->sms);
+    p.kchunk = k > 0 ? k : span;
+    p.nchunks = (span + p.kchunk - 1) / p.kchunk;
+  }
+  p.prepass = p.prepass && p.nchunks == 1;
+  if (d.kchunk < 0 && ring == 0 && p.ysplit == 1 && !p.prepass && take_wide(L.nx, L.ndim == 3, nblk * p.nchunks, c->sms)) {
+    p.wide = true;
+    if (L.nx == 16) p.ysplit = 2;
+  }
+  return p;
+}
+
 // One stage launch.  ring > 0: the telescoping form that also updates that
 // many guard cells around the interior, from Uin's own guard cells.
 // range_first >= 0: `list` is the identity list of blocks [range_first,
@@ -247,34 +291,12 @@ int stage_launch(gbh_ctx* c, const double* Uin, const double* Un, double* Uout, 
   A.smax_acc = dt_epilogue ? c->d_smax : nullptr;
   A.floor_count = c->d_words + 1;
   A.problem = c->d_problem;
-  A.ysplit = (ring == 0 || ring == 2 || ring == 4) ? c->ysplit[ring / 2] : 1;
-  // The face pre-pass by default only below 16 cells per side: a block of 16^3
-  // has few boundary faces for what the extra launch and its buffer cost now
-  // that a face takes 19 FP64 instructions (4096 blocks of 16^3: 12.32 ms a step
-  // with it, 12.17 without; 4096 blocks of 8^3: 1.86 and 2.09).
-  const bool prepass = c->face_prepass && c->d_bflux && ring == 0 && gather && (!list || range_first >= 0) &&
-                       A.ysplit == 1 && (c->prepass_asked || c->lay.nx < 16);
-  if (c->lay.ndim == 3) {
-    // a ring-updating stage spans nz + 2*ring planes; with the pre-pass a work item
-    // is a whole block: where the caller asked for it, and in every range of a
-    // pipelined stage (a later range reads faces that an earlier one solved)
-    const int span = c->lay.nz + 2 * ring;
-    const int side = c->lay.nx + 2 * ring;
-    const long long nblk = list ? nlist : c->refined ? c->nactive : c->lay.nblocks;
-    int k = c->kchunk;
-    if (k < 0)
-      k = prepass && (range_first >= 0 || c->prepass_asked) ? span
-                                                            : auto_kchunk(span, nblk, side * side / A.ysplit, c->sms);
-    A.kchunk = k > 0 ? k : span;
-    A.nchunks = (span + A.kchunk - 1) / A.kchunk;
-  }
-  const long long items = (list ? nlist : c->refined ? c->nactive : c->lay.nblocks) * (long long)A.nchunks;
-  if (c->kchunk < 0 && ring == 0 && A.ysplit == 1 && !(prepass && A.nchunks == 1) &&
-      take_wide(c->lay.nx, c->lay.ndim == 3, items, c->sms)) {
-    A.wide = 1;
-    if (c->lay.nx == 16) A.ysplit = 2;
-  }
-  A.items_per_cta = c->items_per_cta;
+  const StagePlan p = plan_stage(c, ring, gather, list ? nlist : 0, list != nullptr, range_first >= 0);
+  A.kchunk = p.kchunk;
+  A.nchunks = p.nchunks;
+  A.items_per_cta = p.items_per_cta;
+  A.ysplit = p.ysplit;
+  A.wide = p.wide;
   if (c->refined) {
     A.block_list = c->d_active;
     A.nlist = c->nactive;
@@ -289,7 +311,7 @@ int stage_launch(gbh_ctx* c, const double* Uin, const double* Un, double* Uout, 
   cudaEvent_t stop;
   int rc = record_start(c, s, &stop);
   if (rc) return rc;
-  if (prepass && A.nchunks == 1) {
+  if (p.prepass) {
     // each block face solved once, then read by the stage
     const int lo = list ? range_first : 0, hi = list ? range_first + nlist : -1;
     if ((rc = cuda_err(c, gbh::launch_face_fluxes(A, c->d_bflux, s, lo, hi), "face pre-pass launch"))) return rc;
@@ -989,86 +1011,65 @@ int gbh_autotune(gbh_ctx* c, const double* U, int* kchunk_out, int* items_out, v
   if (rc) return rc;
   if (!U || !aligned8(U)) return set_err(c, GBH_ERR_INVAL, "null or misaligned state pointer");
   cudaStream_t s = (cudaStream_t)stream;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+    if (e0) cudaEventDestroy(e0);
+    return set_err(c, GBH_ERR_CUDA, "cudaEventCreate failed");
+  }
   const bool timing = c->timing;
   c->timing = false;
   drop_graph(c);
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const Decomp held[3] = {c->dec[0], c->dec[1], c->dec[2]};
   std::vector<int> kcs = {0};
   if (c->lay.ndim == 3 && c->lay.nz >= 8 && c->lay.nz % 2 == 0) kcs.push_back(c->lay.nz / 2);
   std::vector<int> splits = {1};
   if (c->lay.nx >= 8) splits.push_back(2);
   const long long nlist = c->refined ? c->nactive : c->lay.nblocks;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
-    return set_err(c, GBH_ERR_CUDA, "cudaEventCreate failed");
-  // the interior stage: z-chunk x CTAs' items x row bands (an unsplit tile
-  // keeps two CTAs per SM resident, a band four)
-  float best = 1e30f;
-  int best_kc = 0, best_ipc = 1, best_split = 1;
-  if (c->lay.ndim == 2) {
-    // first what a launch chooses by itself (wide CTAs on a small lattice)
-    best_kc = c->kchunk = -1;
-    c->items_per_cta = 1;
-    c->ysplit[0] = 1;
-    rc = time_stage(c, U, 0, e0, e1, s, &best);
-  }
-  for (int split : splits) {
-    if (rc) break;
+  // first what a launch chooses by itself, the default of a new context; a fixed
+  // choice has to be 2% faster, about what two timed launches can tell apart
+  auto tune = [&](int ring, const std::vector<Decomp>& fixed) {
+    Decomp& d = c->dec[ring / 2];
+    Decomp pick;
+    d = pick;
+    float best = 0.f, ms = 0.f;
+    if ((rc = time_stage(c, U, ring, e0, e1, s, &best))) return;
+    best *= 0.98f;
+    for (const Decomp& t : fixed) {
+      d = t;
+      if ((rc = time_stage(c, U, ring, e0, e1, s, &ms))) return;
+      if (ms < best) {
+        best = ms;
+        pick = t;
+      }
+    }
+    d = pick;
+  };
+  // the interior stage: z-chunk x a CTA's items x row bands, the last count of items
+  // that of a CTA where each SM holds as many as fit on it
+  std::vector<Decomp> fixed;
+  for (int split : splits)
     for (int kc : kcs) {
       const long long nitems = nlist * (kc > 0 ? (c->lay.nz + kc - 1) / kc : 1) * split;
-      const long long resident = 2LL * split * sms;
-      const long long persistent = (nitems + resident - 1) / resident;
-      std::vector<int> ipcs = {1, 2, 4};
-      if (persistent > 4) ipcs.push_back((int)persistent);
-      for (int ipc : ipcs) {
-        c->kchunk = kc;
-        c->items_per_cta = ipc;
-        c->ysplit[0] = split;
-        float ms = 0.f;
-        if ((rc = time_stage(c, U, 0, e0, e1, s, &ms))) break;
-        if (ms < best) {
-          best = ms;
-          best_kc = kc;
-          best_ipc = ipc;
-          best_split = split;
-        }
-      }
-      if (rc) break;
+      const long long resident = (long long)gbh::stage_ctas_per_sm(c->lay.nx, c->lay.ndim, split) * c->sms;
+      const long long persistent = resident > 0 ? (nitems + resident - 1) / resident : 0;
+      for (int ipc : {1, 2, 4}) fixed.push_back({kc, ipc, split});
+      if (persistent > 4) fixed.push_back({kc, (int)persistent, split});
     }
-    if (rc) break;
-  }
-  c->kchunk = best_kc;
-  c->items_per_cta = best_ipc;
-  c->ysplit[0] = best_split;
+  tune(0, fixed);
   // the ring stages of the telescoping mode (ring 2; and 4 with three
-  // stages): row bands with the decomposition chosen above, on U's own guard
-  // cells as they are (the time does not depend on their values)
-  if (!rc && c->telescoping) {
-    for (int ring = 2; ring <= 2 * (c->nstages - 1) && !rc; ring += 2) {
-      if (c->lay.g < ring + 2) continue;
-      float best_r = 1e30f;
-      int pick = 1;
-      for (int split : splits) {
-        c->ysplit[ring / 2] = split;
-        float ms = 0.f;
-        if ((rc = time_stage(c, U, ring, e0, e1, s, &ms))) break;
-        if (ms < best_r) {
-          best_r = ms;
-          pick = split;
-        }
-      }
-      c->ysplit[ring / 2] = pick;
-    }
-  }
+  // stages) by the same list, on U's own guard cells as they are (the time does
+  // not depend on their values)
+  for (int ring = 2; !rc && c->telescoping && ring <= 2 * (c->nstages - 1); ring += 2)
+    if (c->lay.g >= ring + 2) tune(ring, fixed);
+  if (rc)
+    for (int r = 0; r < 3; ++r) c->dec[r] = held[r];
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   c->timing = timing;
   cudaMemsetAsync(c->d_words + 1, 0, sizeof(unsigned long long), s);   // trial launches may count floors
   if (rc) return rc;
-  if (kchunk_out) *kchunk_out = best_kc > 0 ? best_kc : c->lay.nz;
-  if (items_out) *items_out = best_ipc;
+  if (kchunk_out) *kchunk_out = c->dec[0].kchunk > 0 ? c->dec[0].kchunk : c->lay.nz;
+  if (items_out) *items_out = c->dec[0].items_per_cta;
   return GBH_OK;
 }
 
@@ -1079,7 +1080,8 @@ int gbh_set_tile_split(gbh_ctx* c, int ring, int ysplit) {
     return set_err(c, GBH_ERR_INVAL, "ysplit must be 1, or 2 for blocks of at least 8 cells per side (got %d)",
                    ysplit);
   drop_graph(c);
-  c->ysplit[ring / 2] = ysplit;
+  c->dec[ring / 2].ysplit = ysplit;
+  if (ring == 0) c->dec_range.ysplit = ysplit;
   return GBH_OK;
 }
 
@@ -1087,7 +1089,7 @@ int gbh_get_tile_split(gbh_ctx* c, int ring, int* ysplit) {
   if (!c) return set_err(nullptr, GBH_ERR_INVAL, "null context");
   if (ring != 0 && ring != 2 && ring != 4) return set_err(c, GBH_ERR_INVAL, "ring must be 0, 2 or 4 (got %d)", ring);
   if (!ysplit) return set_err(c, GBH_ERR_INVAL, "null output pointer");
-  *ysplit = c->ysplit[ring / 2];
+  *ysplit = c->dec[ring / 2].ysplit;
   return GBH_OK;
 }
 
@@ -1189,11 +1191,34 @@ int gbh_get_prim_carry(gbh_ctx* c, int* enabled) {
 
 int gbh_set_decomposition(gbh_ctx* c, int kchunk, int items_per_cta) {
   if (!c) return set_err(nullptr, GBH_ERR_INVAL, "null context");
-  if (items_per_cta < 1 || kchunk < 0 || (kchunk > 0 && (c->lay.ndim != 3 || kchunk < 2 || kchunk > c->lay.nz)))
+  if (items_per_cta < 1 || kchunk < -1 || (kchunk > 0 && (c->lay.ndim != 3 || kchunk > c->lay.nz)))
     return set_err(c, GBH_ERR_INVAL, "invalid decomposition (kchunk %d, items per CTA %d)", kchunk, items_per_cta);
   drop_graph(c);
-  c->kchunk = (kchunk == c->lay.nz) ? 0 : kchunk;
-  c->items_per_cta = items_per_cta;
+  for (Decomp* d : {&c->dec[0], &c->dec[1], &c->dec[2], &c->dec_range}) {
+    d->kchunk = kchunk == c->lay.nz ? 0 : kchunk;
+    d->items_per_cta = items_per_cta;
+  }
+  return GBH_OK;
+}
+
+int gbh_get_decomposition(gbh_ctx* c, int* kchunk, int* items_per_cta) {
+  if (!c) return set_err(nullptr, GBH_ERR_INVAL, "null context");
+  if (!kchunk || !items_per_cta) return set_err(c, GBH_ERR_INVAL, "null output pointer");
+  *kchunk = c->dec[0].kchunk;
+  *items_per_cta = c->dec[0].items_per_cta;
+  return GBH_OK;
+}
+
+int gbh_stage_plan(gbh_ctx* c, int ring, int* plan) {
+  if (!c) return set_err(nullptr, GBH_ERR_INVAL, "null context");
+  if (ring != 0 && ring != 2 && ring != 4) return set_err(c, GBH_ERR_INVAL, "ring must be 0, 2 or 4 (got %d)", ring);
+  if (!plan) return set_err(c, GBH_ERR_INVAL, "null output pointer");
+  const StagePlan p = plan_stage(c, ring, ring == 0 && !c->telescoping, 0, false, false);
+  plan[0] = p.kchunk;
+  plan[1] = p.items_per_cta;
+  plan[2] = p.ysplit;
+  plan[3] = p.wide;
+  plan[4] = p.prepass;
   return GBH_OK;
 }
 

@@ -143,7 +143,7 @@ void layout_from_params(const gbh_params* p, Layout* L, Eos* e);
 void face_table_from_params(const gbh_params* p, long long b, int face[6], double inv_dx[3]);
 void stage_args_common(StageArgs* A, const Layout& L, const Eos& e);
 int set_create_error(int code, const char* msg);
-size_t stage_smem_bytes(int nx);
+int stage_ctas_per_sm(int nx, int ndim, int ysplit);   // of the interior stage; 0: unknown
 cudaError_t stage_prepare(int nx, int ndim);  // opt-in to the dynamic shared memory size
 
 struct FillArgs {

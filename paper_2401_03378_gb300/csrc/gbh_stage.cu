@@ -780,6 +780,16 @@ cudaError_t prepare_one() {
                               (int)smem_for<N, E, S, fluxes_over_prims<N, E, S, WIDE>()>());
 }
 
+// CTAs of the interior stage that fit on an SM (0: unknown).
+template <int N, bool D3, int S>
+int resident_t() {
+  int n = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &n, stage_kernel<N, D3, 0, S>, stage_threads<N, 0, S>(), smem_for<N, 0, S, fluxes_over_prims<N, 0, S, false>()>());
+  if (e != cudaSuccess) cudaGetLastError();   // not an error of the caller's
+  return e == cudaSuccess ? n : 0;
+}
+
 // The row-band split (S = 2) exists for N >= 8 (a band of at least 4 rows).
 template <int N, bool D3>
 cudaError_t prepare_t() {
@@ -828,11 +838,14 @@ cudaError_t launch_e(const StageArgs& a, cudaStream_t s) {
 
 GBH_CHECK_TAKE(check_take_stage)
 
-size_t stage_smem_bytes(int nx) {
+int stage_ctas_per_sm(int nx, int ndim, int ysplit) {
+  const bool d3 = ndim == 3;
   switch (nx) {
-    case 4: return smem_for<4, 0, 1>();
-    case 8: return smem_for<8, 0, 1>();
-    case 16: return smem_for<16, 0, 1>();
+    case 4: return ysplit != 1 ? 0 : d3 ? resident_t<4, true, 1>() : resident_t<4, false, 1>();
+    case 8: return ysplit == 2 ? (d3 ? resident_t<8, true, 2>() : resident_t<8, false, 2>())
+                               : (d3 ? resident_t<8, true, 1>() : resident_t<8, false, 1>());
+    case 16: return ysplit == 2 ? (d3 ? resident_t<16, true, 2>() : resident_t<16, false, 2>())
+                                : (d3 ? resident_t<16, true, 1>() : resident_t<16, false, 1>());
     default: return 0;
   }
 }

@@ -212,12 +212,28 @@ class Hydro:
         return U
 
     def autotune(self, U):
+        """Keep the default work decomposition or a fixed one that is faster on U;
+        returns (z planes per work item, nz for the default too; items per CTA)."""
         kc, ipc = C.c_int(0), C.c_int(0)
         self._check(self.lib.gbh_autotune(self.ctx, self._state(U), C.byref(kc), C.byref(ipc), _stream_handle()))
         return int(kc.value), int(ipc.value)
 
-    def set_decomposition(self, kchunk: int, items_per_cta: int):
+    def set_decomposition(self, kchunk: int, items_per_cta: int = 1):
+        """z planes per work item (0: whole blocks; -1: picked per launch, as in a new
+        context) and work items per CTA of every stage."""
         self._check(self.lib.gbh_set_decomposition(self.ctx, int(kchunk), int(items_per_cta)))
+
+    def decomposition(self):
+        """(kchunk, items_per_cta) of the interior stage, as set_decomposition takes them."""
+        kc, ipc = C.c_int(0), C.c_int(0)
+        self._check(self.lib.gbh_get_decomposition(self.ctx, C.byref(kc), C.byref(ipc)))
+        return int(kc.value), int(ipc.value)
+
+    def stage_plan(self, ring: int = 0) -> dict:
+        """What a stage of that ring width over all blocks takes with the settings as they are."""
+        p = (C.c_int * 5)()
+        self._check(self.lib.gbh_stage_plan(self.ctx, int(ring), p))
+        return {"kchunk": p[0], "items_per_cta": p[1], "ysplit": p[2], "wide": bool(p[3]), "face_prepass": bool(p[4])}
 
     def set_tile_split(self, ring: int, ysplit: int):
         """Row bands per plane tile of the stage kernel for ring width 0, 2 or 4."""
