@@ -230,30 +230,14 @@ def host_cpu_model():
 
 
 def autotuned(h, U, rings, time_default):
-    """Run the library's autotuner on U and describe its choice; when that is
-    not the default decomposition (whole block per work item, one item per
-    CTA, unsplit tiles), time_default() is timed with the default restored
-    before the choice is set back."""
-    kc, ipc = h.autotune(U)
-    splits = {r: h.tile_split(r) for r in rings}
-    full = h.n[2] if h.ndim == 3 else 1
-    choice = {"kchunk": kc, "items_per_cta": ipc, "ysplit": {str(r): s for r, s in splits.items()}}
-    is_default = kc == full and ipc == 1 and all(s == 1 for s in splits.values())
-    out = {"chosen": choice, "chosen_is_default": is_default, "default_ms_per_step": None}
-    if not is_default:
-        h.set_decomposition(0, 1)
-        for r in rings:
-            h.set_tile_split(r, 1)
-        out["default_ms_per_step"] = time_default()
-        h.set_decomposition(kc if h.ndim == 3 else 0, ipc)
-        for r, sp in splits.items():
-            h.set_tile_split(r, sp)
-    return out
-
-
-def lat_kchunk(lat):
-    """z planes of one work item in the default decomposition (the whole block)."""
-    return lat.n[2] if lat.ndim == 3 else 1
+    """Time the context as it is new (the decomposition picked per launch), then run
+    the library's autotuner on U and describe its choice per ring width."""
+    default_ms = time_default()
+    before = {r: h.stage_plan(r) for r in rings}
+    h.autotune(U)
+    after = {r: h.stage_plan(r) for r in rings}
+    return {"chosen": {str(r): p for r, p in after.items()}, "chosen_is_default": after == before,
+            "default_ms_per_step": default_ms}
 
 
 def make_problem(nb: int):
@@ -263,9 +247,8 @@ def make_problem(nb: int):
 
 
 def prepass_runs(h):
-    """Whether the stages of a context with default settings launch the face pre-pass
-    (by default only for blocks narrower than 16 cells)."""
-    return h.face_prepass() and h.n[0] < 16
+    """Whether the halo-gathering stages of a context launch the face pre-pass."""
+    return h.stage_plan()["face_prepass"]
 
 
 def fp64_probe_tflops(gb, torch, form=1):
@@ -592,6 +575,7 @@ def run_two_level(args, gb, torch, barrier):
     barrier()
     secs = e0.elapsed_time(e1) / 1e3
     nbad = h.check_state(U)
+    pre = 2 if prepass_runs(h) else 0     # the face pre-pass of the two all-levels stages
     # the same grid in the level-by-level telescoping variant
     h.set_telescoping(True)
     U.copy_(torch.from_numpy(U0))
@@ -606,7 +590,6 @@ def run_two_level(args, gb, torch, barrier):
     barrier()
     tsecs = e0.elapsed_time(e1) / 1e3
     tbad = h.check_state(U)
-    pre = 2 if prepass_runs(h) else 0     # the face pre-pass of the two all-levels stages
     h.close()
     del U
     torch.cuda.empty_cache()
@@ -656,7 +639,7 @@ def run_ensemble(args, gb, torch, barrier):
         return ms
 
     tuning = autotuned(h, U, (0,), default_ms) if args.autotune else None
-    kc, ipc = (tuning["chosen"]["kchunk"], tuning["chosen"]["items_per_cta"]) if tuning else (lat_kchunk(lats[0]), 1)
+    plan = h.stage_plan()
     dt = h.compute_dt(U)
     h.advance_graph(U, n, dt)          # capture + warm-up run
     U.copy_(torch.from_numpy(U0))
@@ -683,7 +666,7 @@ def run_ensemble(args, gb, torch, barrier):
                         "noise (sigma 0.1, seeds 1000+i), own CFL dt each, FP64",
             "zones": zones, "blocks": sum(l.nblocks for l in lats), "steps": n,
             "batched_graph": {"value": zones * n / batched, "unit": UNIT, "ms_per_step": 1e3 * batched / n,
-                              "launches_per_step": 3, "graph_launches": 1, "kchunk": kc, "items_per_cta": ipc,
+                              "launches_per_step": 3, "graph_launches": 1, "stage_plan": plan,
                               "autotune": tuning},
             "one_launch_per_problem": {"value": zones * n / separate, "unit": UNIT,
                                        "ms_per_step": 1e3 * separate / n, "launches_per_step": 3 * len(lats)},
