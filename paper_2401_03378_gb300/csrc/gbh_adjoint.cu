@@ -115,7 +115,6 @@ __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double W
   // ---- forward ----
   // From the densities and pressures to the sound speeds and Roe weights, and
   // the quotients S* and t, as in hllc_flux: Wide numbers on the integer pipes.
-  uint32_t bad = non_finite_mask(WL, WR);
   const Wide RL = wide_of(rL), RR = wide_of(rR);
   const Wide P = wide_mul(RL, RR), iP = wide_rcp(P), sP = wide_sqrt(P);
   const Wide IL = wide_mul(RR, iP), IR = wide_mul(RL, iP);   // 1/rho
@@ -123,9 +122,8 @@ __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double W
   const Wide CL = wide_sqrt(CL2), CR = wide_sqrt(CR2);
   const Wide D = wide_rcp_low(wide_add(sP, RR));
   const Wide XL = wide_mul(sP, D), XR = wide_mul(RR, D);     // Roe weights
-  // these can leave the range of a double; a 1/rho that does leaves no gradient
+  // these can leave the range of a double
   const double iL = wide_signed(IL, 0u), iR = wide_signed(IR, 0u);
-  bad |= IL.e < 1 || IR.e < 1 ? 0x7fffffffu : 0u;
   const double cL2 = wide_signed(CL2, 0u), cR2 = wide_signed(CR2, 0u);
   const double cL = wide_double(CL), cR = wide_double(CR);
   const double qL = wide_double(wide_rcp(wide_of(cL))), qR = wide_double(wide_rcp(wide_of(cR)));   // 1/c
@@ -149,7 +147,8 @@ __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double W
   const Wide RD = wide_rcp(wide_add(ML, MR));              // -1 / (mL - mR)
   const double rd = wide_signed(RD, 0x80000000u);
   const double num = fma(-mR, uR, fma(mL, uL, S(pR, pL)));
-  bad |= overflow_mask(du2, num);
+  uint32_t bad = no_flux_mask(WL, WR, du2, num);
+  bad |= IL.e < 1 || IR.e < 1 ? 0x7fffffffu : 0u;          // a 1/rho below the range leaves no gradient
   const Wide WS = wide_mul(wide_of0(num), RD);
   const uint32_t ssgn = sign01(num) ^ 1u;
   const double Ss = wide_signed(WS, ssgn << 31 | bad);

@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(kThreads) dt_reduce_kernel(const DtArgs a, con
       for (int v = 0; v < 5; ++v) U[v] = __ldg(src + o + v * L.vstride);
       Wide ir;
       cons_to_prim_ir(U, W, e, ir);
+      prim_beyond(U, W, ir, e);
       smax = max_nonneg(smax, signal_speed_ir(W, ir, e, ix, iy, iz, isum, d3));
     }
     if (problem) {

@@ -68,33 +68,35 @@ __device__ __forceinline__ uint32_t sign01(double x) { return hi_word(x) >> 31; 
 // Infinity or NaN.
 __device__ __forceinline__ bool not_finite(double x) { return (hi_word(x) & 0x7ff00000u) == 0x7ff00000u; }
 
-// A NaN's high word where one of two sums of finite terms overflowed, else 0.
-__device__ __forceinline__ uint32_t overflow_mask(double a, double b) {
-  return not_finite(a) || not_finite(b) ? 0x7fffffffu : 0u;
-}
+// z + 0 where x is finite and below 2^1017 in magnitude, else NaN: FP32 arithmetic on
+// the high word, whose exponent field is all ones from there.  One instruction of
+// the otherwise idle FP32 pipe; callers look closer where the sum is not +0.
+__device__ __forceinline__ float watch(double x, float z) { return fmaf(__uint_as_float(hi_word(x)), 0.0f, z); }
 
-// See hllc_flux.
-__device__ __forceinline__ uint32_t non_finite_mask(const double WL[5], const double WR[5]) {
-  float z = 0.0f;
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    z = fmaf(__uint_as_float(hi_word(WL[v])), 0.0f, z);
-    z = fmaf(__uint_as_float(hi_word(WR[v])), 0.0f, z);
-  }
-  return __float_as_uint(z);
+// A NaN's high word where a face has no flux, else 0.  Not finite: a density or
+// pressure, the squared velocity jump (which a velocity that is not makes so) or the
+// contact speed's numerator; the unpacked form would take them as numbers.  Without a
+// branch, which would keep the two halves of the face from being scheduled together
+// (1.2% of a step).
+__device__ __forceinline__ uint32_t no_flux_mask(const double WL[5], const double WR[5], double du2, double num) {
+  auto larger = [](uint32_t a, uint32_t b) { return a > b ? a : b; };
+  const uint32_t rho = larger(hi_word(WL[0]), hi_word(WR[0])), p = larger(hi_word(WL[4]), hi_word(WR[4]));
+  const uint32_t top = larger(larger(rho, p), larger(hi_word(du2), hi_word(num) & 0x7fffffffu));
+  return top >= 0x7ff00000u ? 0x7fffffffu : 0u;
 }
 
 // calcEos role: conserved (rho, mx, my, mz, E) -> primitive (rho, u, v, w, p),
 // p = (gamma-1) (E - (mx^2 + my^2 + mz^2) / (2 rho)).  Floors rho at small_rho and
 // p at small_p (floored_rho, floored_p) and leaves 1/rho in ir.  On the integer pipes but
 // for the subtraction: 8 FP64 instructions of 64 cycles became 1 and about 110
-// more integer ones; a NaN or infinity in any of the five reaches u, v, w and p through
-// the FP32 mask.
+// more integer ones.  A conserved variable that is not finite, or beyond 2^1017, makes u,
+// v and w NaN, and p NaN or the floor (through the FP32 watch: exact tests took 0.5% of a
+// step); prim_beyond gives what the plain formulas do there.
 __device__ __forceinline__ void cons_to_prim_flags(const double U[5], double W[5], const Eos& e, Wide& ir,
                                                    bool& floored_rho, bool& floored_p) {
   float z = 0.0f;
 #pragma unroll
-  for (int v = 0; v < 5; ++v) z = fmaf(__uint_as_float(hi_word(U[v])), 0.0f, z);
+  for (int v = 0; v < 5; ++v) z = watch(U[v], z);
   const uint32_t bad = __float_as_uint(z);
   double rho = U[0];
   floored_rho = less_d(rho, e.small_rho);
@@ -110,6 +112,21 @@ __device__ __forceinline__ void cons_to_prim_flags(const double U[5], double W[5
   floored_p = less_d(p, e.small_p);
   if (floored_p) p = e.small_p;
   W[0] = rho; W[1] = u; W[2] = v; W[3] = w; W[4] = p;
+}
+
+// W of cons_to_prim_flags where a velocity is not finite, by the plain FP64 formulas:
+// an infinite momentum is an infinite velocity at the pressure floor, and numbers beyond
+// 2^1017 are numbers.  For the CFL speed of given states (dt = 0 beside an infinite
+// momentum).
+__device__ __forceinline__ void prim_beyond(const double U[5], double W[5], const Wide& ir, const Eos& e) {
+  if (!not_finite(W[1]) && !not_finite(W[2]) && !not_finite(W[3])) return;
+  const double r = not_finite(W[0]) ? bitsd(0x7ff8000000000000LL) : wide_signed(ir, 0u);
+#pragma unroll
+  for (int v = 1; v < 4; ++v) W[v] = mul(U[v], r, e.k);
+  const double m2 = fma(U[3], W[3], fma(U[2], W[2], mul(U[1], W[1], e.k)));
+  const double p = mul(e.gm1, fma(-0.5, m2, U[4]), e.k);
+  const bool nan = mag_key(p) > mag_key(bitsd(0x7ff0000000000000LL));
+  W[4] = nan ? bitsd(0x7ff8000000000000LL) : less_d(p, e.small_p) ? e.small_p : p;
 }
 
 // The same; returns 1 when a floor applied.
@@ -252,11 +269,6 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
   const double rL = WL[0], uL = WL[1], vL = WL[2], wL = WL[3], pL = WL[4];
   const double rR = WR[0], uR = WR[1], vR = WR[2], wR = WR[3], pR = WR[4];
 
-  // +0, or a NaN's bits when any input is not finite (FP32 arithmetic on the
-  // high words, whose exponent field is all ones for an infinity, a NaN or a
-  // magnitude from 2^1017): OR-ed into S* and t, from where it reaches every flux
-  uint32_t bad = non_finite_mask(WL, WR);
-
   // the wave speeds' positive part, on the integer pipes
   const Wide RL = wide_of(rL), RR = wide_of(rR);
   const Wide P = wide_mul(RL, RR);
@@ -283,7 +295,7 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
   const double mL = wide_signed(ML, 0x80000000u), mR = wide_signed(MR, 0u);
   // S* = num / (m_L - m_R) = -num / (|m_L| + |m_R|)
   const double num = fma(-mR, uR, fma(mL, uL, sub(pR, pL, k)));
-  bad |= overflow_mask(du2_d, num);                        // which the unpacked form would take as 2^1024
+  const uint32_t bad = no_flux_mask(WL, WR, du2_d, num);   // OR-ed into S* and t, from where it reaches every flux
   const Wide WS = wide_mul(wide_of0(num), wide_rcp(wide_add(ML, MR)));
   const uint32_t ssgn = sign01(num) ^ 1u;
   const double Ss = wide_signed(WS, ssgn << 31 | bad);

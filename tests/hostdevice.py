@@ -48,13 +48,16 @@ void hd_hllc(const double* q, long n, const double* WL, const double* WR, double
   const Eos e = eos(q);
   for (long i = 0; i < 5 * n; i += 5) hllc_flux(WL + i, WR + i, e, F + i);
 }
-// W, the floor count and the CFL speed for inverse cell widths d
-void hd_prim(const double* q, long n, const double* U, const double* d, double* W, int* hit, double* speed) {
+// W and the floor count of a stage; W as the CFL reduction takes it and its speed for
+// inverse cell widths d
+void hd_prim(const double* q, long n, const double* U, const double* d, double* W, int* hit, double* Wd, double* speed) {
   const Eos e = eos(q);
   for (long i = 0; i < n; ++i) {
     Wide ir;
     hit[i] = cons_to_prim_ir(U + 5 * i, W + 5 * i, e, ir);
-    speed[i] = signal_speed_ir(W + 5 * i, ir, e, d[0], d[1], d[2], inv_width_sum(e, d[0], d[1], d[2], true), true);
+    std::memcpy(Wd + 5 * i, W + 5 * i, 5 * sizeof(double));
+    prim_beyond(U + 5 * i, Wd + 5 * i, ir, e);
+    speed[i] = signal_speed_ir(Wd + 5 * i, ir, e, d[0], d[1], d[2], inv_width_sum(e, d[0], d[1], d[2], true), true);
   }
 }
 // s / (s + b) with s = sqrt(a): the Roe weight's form, from the unpacked numbers
@@ -101,12 +104,14 @@ class HostDevice:
         self.lib.hd_hllc(_p(self.q), C.c_long(len(WL)), _p(WL), _p(WR), _p(F))
         return F
 
-    def prim(self, U, inv_dx=(1.0, 2.0, 3.0)):
+    def prim(self, U, inv_dx=(1.0, 2.0, 3.0), beyond=False):
+        """(W, floor count, CFL speed); beyond: W as the CFL reduction takes it."""
         U = np.ascontiguousarray(np.atleast_2d(U), dtype=np.float64)
         d = np.array(inv_dx, dtype=np.float64)
-        W, hit, s = np.empty_like(U), np.empty(len(U), dtype=np.int32), np.empty(len(U))
-        self.lib.hd_prim(_p(self.q), C.c_long(len(U)), _p(U), _p(d), _p(W), _p(hit), _p(s))
-        return W, hit, s
+        W, Wd = np.empty_like(U), np.empty_like(U)
+        hit, s = np.empty(len(U), dtype=np.int32), np.empty(len(U))
+        self.lib.hd_prim(_p(self.q), C.c_long(len(U)), _p(U), _p(d), _p(W), _p(hit), _p(Wd), _p(s))
+        return (Wd if beyond else W), hit, s
 
     def weight(self, a, b):
         a, b = (np.ascontiguousarray(x, dtype=np.float64) for x in (a, b))

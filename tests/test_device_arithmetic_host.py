@@ -82,3 +82,61 @@ def test_the_kinetic_energy_overflow_of_a_cell(dev):
             assert s[0] >= abs(m) and np.isfinite(s[0])
     W, hit, s = dev.prim([1e-100, 1e300, 0.0, 0.0, 1.0])
     assert W[0, 1] == np.inf and W[0, 4] == 1e-300 and s[0] == np.inf
+
+
+# beyond 2^1017, where the FP32 watch on the high words takes a number for an infinity
+BEYOND = [[1.0, 0.0, 0.0, 0.0, 1e307], [1e306, 1e290, -1e290, 1e280, 1.7e308], [1e307, 1.0, 0.0, 0.0, 1.0],
+          [1e307, 1e307, 0.0, 0.0, 1e307], [1.0, 1e300, 0.0, 0.0, 1e307], [1e306, 1e300, -1.7e308, 1e290, 1.7e308],
+          [1e-100, 0.0, 2e306, 0.0, 1.0]]
+
+
+@pytest.mark.parametrize("U", BEYOND)
+def test_finite_states_beyond_2_to_the_1017(dev, U):
+    """The CFL speed of finite states of any magnitude is that of the plain FP64
+    formulas; a stage takes them for non-finite ones."""
+    W, hit, s = dev.prim(U, inv_dx=(0.5, 0.25, 0.125), beyond=True)
+    with np.errstate(over="ignore"):
+        u = np.array(U[1:4]) / U[0]
+        p = 0.4 * (U[4] - 0.5 * np.dot(U[1:4], u))
+        c = np.sqrt(1.4 * max(p, 1e-300) / U[0])
+        ref = c * 0.875 + np.abs(u) @ [0.5, 0.25, 0.125]
+    assert W[0, 0] == U[0] and np.allclose(W[0, 1:4], u, rtol=4e-16, atol=0)
+    assert W[0, 4] == 1e-300 if not p >= 1e-300 else abs(W[0, 4] / p - 1) < 1e-15
+    assert s[0] == ref or abs(s[0] / ref - 1) < 1e-14
+    assert np.all(np.isnan(dev.prim(U)[0][0, 1:4]))
+
+
+@pytest.mark.parametrize("u", [0.0, 0.5, -0.25])
+def test_a_flux_at_pressures_beyond_2_to_the_1017(dev, u):
+    W = np.array([1.0, u, 0.1, 0.0, 1e307])
+    ref, got = orc.hllc(W, W), dev.hllc(W, W)[0]
+    assert np.all(np.isfinite(got)) and np.max(np.abs(got - ref)) <= 1e-13 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("k,x", [(k, x) for k in range(5) for x in (np.inf, -np.inf, np.nan)])
+def test_a_non_finite_variable_of_a_cell(dev, k, x):
+    """In a stage it makes the velocities NaN.  For the CFL speed an infinite momentum is an infinite velocity (dt = 0) at the
+    pressure floor, and a NaN stays a NaN."""
+    for E in (2.5, -2.5, 1e-3):
+        U = np.array([1.0, 0.3, -0.2, 0.1, E])
+        U[k] = x
+        V, _, s = dev.prim(U)
+        assert np.all(np.isnan(V[0, 1:4])) and (np.isnan(V[0, 4]) or V[0, 4] == 1e-300)
+        W, _, _ = dev.prim(U, beyond=True)
+        if 1 <= k <= 3 and np.isinf(x):
+            assert W[0, k] == x and W[0, 4] == 1e-300 and s[0] == np.inf
+            assert np.allclose(np.delete(W[0, 1:4], k - 1), np.delete(U[1:4], k - 1), rtol=1e-15)
+        elif np.isnan(x):
+            assert np.isnan(W[0, 4]) and np.isnan(s[0]) and (np.isnan(W[0, k]) or k == 0)
+        elif k == 4:
+            assert np.array_equal(W[0, :4], U[:4]) and W[0, 4] == (np.inf if x > 0 else 1e-300)
+        elif x > 0:
+            assert np.isnan(W[0, 4]) and np.isnan(s[0])
+
+
+@pytest.mark.parametrize("v", range(5))
+@pytest.mark.parametrize("x", [np.inf, -np.inf, np.nan])
+def test_a_non_finite_face_state_has_no_flux(dev, v, x):
+    a, b = np.array([1.0, 0.3, 0.1, 0.0, 1.0]), np.array([0.5, 0.2, 0.0, 0.1, 0.7])
+    a[v] = x
+    assert np.all(np.isnan(dev.hllc(a, b))) and np.all(np.isnan(dev.hllc(b, a)))

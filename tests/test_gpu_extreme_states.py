@@ -68,3 +68,21 @@ def test_scaled_states(gb, k):
     (a, la), (b, lb) = res
     assert np.max(np.abs(a - b)) <= 1e-13 * np.max(np.abs(a))
     assert np.max(np.abs(la - lb)) <= 1e-12 * np.max(np.abs(la))
+
+
+@pytest.mark.parametrize("ndim,var", [(2, 1), (2, 2), (3, 1), (3, 2), (3, 3)])
+@pytest.mark.parametrize("x", [np.inf, -np.inf])
+@pytest.mark.parametrize("n", [4, 16])
+def test_an_infinite_momentum_leaves_no_time_step(gb, ndim, var, x, n):
+    lat = wl.lattice_2d(3, 2, n, n, 4) if ndim == 2 else wl.lattice_3d(2, 2, 2, n, n, 6, 4)
+    U = wl.random_state(lat, seed=3, rough=False)
+    U[4, var, lat.gz, 4 + 1, 4 + 2] = x
+    assert float(gb.Hydro.from_lattice(lat).compute_dt(torch.from_numpy(U).cuda())[0]) == 0.0
+
+
+def test_the_time_step_of_a_gas_beyond_2_to_the_1017(gb):
+    lat = wl.lattice_2d(2, 2, 8, 8, 4, bc="periodic")
+    one = np.ones((lat.nblocks,) + lat.padded)
+    U = state(lat, one, 0 * one, 0 * one, 0 * one, 4e306 * one)
+    dt = float(gb.Hydro.from_lattice(lat).compute_dt(torch.from_numpy(U).cuda())[0])
+    assert abs(dt / (0.8 / (2 * np.sqrt(1.4 * 4e306) / lat.dx[0])) - 1.0) <= 1e-14
