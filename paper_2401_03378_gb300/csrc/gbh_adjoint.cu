@@ -144,10 +144,11 @@ __device__ __forceinline__ void hllc_flux_vjp(const double WL[5], const double W
   const Wide DL = wide_of0(dL), DR = wide_of0(dR);
   const Wide ML = wide_mul(RL, DL), MR = wide_mul(RR, DR);
   const double mL = wide_signed(ML, 0x80000000u), mR = wide_signed(MR, 0u);
-  const Wide RD = wide_rcp(wide_add(ML, MR));              // -1 / (mL - mR)
+  const Wide MS = wide_add(ML, MR);
+  const Wide RD = wide_rcp(MS);                            // -1 / (mL - mR)
   const double rd = wide_signed(RD, 0x80000000u);
   const double num = fma(-mR, uR, fma(mL, uL, S(pR, pL)));
-  uint32_t bad = no_flux_mask(WL, WR, du2, num);
+  uint32_t bad = no_flux_mask(WL, WR, du2, num, MS);
   bad |= IL.e < 1 || IR.e < 1 ? 0x7fffffffu : 0u;          // a 1/rho below the range leaves no gradient
   const Wide WS = wide_mul(wide_of0(num), RD);
   const uint32_t ssgn = sign01(num) ^ 1u;

@@ -75,14 +75,17 @@ __device__ __forceinline__ float watch(double x, float z) { return fmaf(__uint_a
 
 // A NaN's high word where a face has no flux, else 0.  Not finite: a density or
 // pressure, the squared velocity jump (which a velocity that is not makes so) or the
-// contact speed's numerator; the unpacked form would take them as numbers.  Without a
-// branch, which would keep the two halves of the face from being scheduled together
-// (1.2% of a step).
-__device__ __forceinline__ uint32_t no_flux_mask(const double WL[5], const double WR[5], double du2, double num) {
+// contact speed's numerator; the unpacked form would take them as numbers.  Zero: the
+// contact speed's denominator m = |m_L| + |m_R|, where both sound speeds are lost in
+// the velocities they are added to (a sum of two products with a zero has an exponent
+// below -5000, any other one above -600).  Without a branch, which would keep the two
+// halves of the face from being scheduled together (1.2% of a step).
+__device__ __forceinline__ uint32_t no_flux_mask(const double WL[5], const double WR[5], double du2, double num,
+                                                 const Wide& m) {
   auto larger = [](uint32_t a, uint32_t b) { return a > b ? a : b; };
   const uint32_t rho = larger(hi_word(WL[0]), hi_word(WR[0])), p = larger(hi_word(WL[4]), hi_word(WR[4]));
   const uint32_t top = larger(larger(rho, p), larger(hi_word(du2), hi_word(num) & 0x7fffffffu));
-  return top >= 0x7ff00000u ? 0x7fffffffu : 0u;
+  return top >= 0x7ff00000u || m.e <= -4096 ? 0x7fffffffu : 0u;
 }
 
 // calcEos role: conserved (rho, mx, my, mz, E) -> primitive (rho, u, v, w, p),
@@ -295,8 +298,9 @@ __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5]
   const double mL = wide_signed(ML, 0x80000000u), mR = wide_signed(MR, 0u);
   // S* = num / (m_L - m_R) = -num / (|m_L| + |m_R|)
   const double num = fma(-mR, uR, fma(mL, uL, sub(pR, pL, k)));
-  const uint32_t bad = no_flux_mask(WL, WR, du2_d, num);   // OR-ed into S* and t, from where it reaches every flux
-  const Wide WS = wide_mul(wide_of0(num), wide_rcp(wide_add(ML, MR)));
+  const Wide MS = wide_add(ML, MR);
+  const uint32_t bad = no_flux_mask(WL, WR, du2_d, num, MS);   // OR-ed into S* and t, from where it reaches every flux
+  const Wide WS = wide_mul(wide_of0(num), wide_rcp(MS));
   const uint32_t ssgn = sign01(num) ^ 1u;
   const double Ss = wide_signed(WS, ssgn << 31 | bad);
 

@@ -140,3 +140,23 @@ def test_a_non_finite_face_state_has_no_flux(dev, v, x):
     a, b = np.array([1.0, 0.3, 0.1, 0.0, 1.0]), np.array([0.5, 0.2, 0.0, 0.1, 0.7])
     a[v] = x
     assert np.all(np.isnan(dev.hllc(a, b))) and np.all(np.isnan(dev.hllc(b, a)))
+
+
+@pytest.mark.parametrize("u", [1e10, -1e10, 3e120, -7e16])
+def test_both_sound_speeds_lost_in_the_velocities(dev, u):
+    """u + c = u - c = u on both sides, where the contact speed is 0 / 0: no flux (NaN),
+    not one of another speed."""
+    for p, q in ((1e-14, 1e-14), (1e-30, 1e-14), (1e-300, 1e-20)):
+        L, R = np.array([1.0, u, 0.1, 0.0, p]), np.array([0.7, u, 0.1, 0.0, q])
+        for a, b in ((L, R), (R, L), (L, L)):
+            assert np.all(np.isnan(dev.hllc(a, b)))
+    # one side's is lost: the flux of the textbook form
+    a, b = np.array([1.0, 1e10, 0.0, 0.0, 1e-14]), np.array([1.0, 1e10, 0.0, 0.0, 1e16])
+    for L, R in ((a, b), (b, a)):
+        ref = orc.hllc(L, R)
+        assert np.max(np.abs(dev.hllc(L, R)[0] - ref)) <= 1e-13 * np.max(np.abs(ref))
+
+
+def test_receding_states_with_both_sound_speeds_lost(dev):
+    L, R = np.array([1.0, -1e10, 0.0, 0.0, 1e-14]), np.array([1.0, 1e10, 0.0, 0.0, 1e-14])
+    assert np.all(np.isnan(orc.hllc(L, R))) and np.all(np.isnan(dev.hllc(L, R)))

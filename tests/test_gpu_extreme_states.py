@@ -86,3 +86,18 @@ def test_the_time_step_of_a_gas_beyond_2_to_the_1017(gb):
     U = state(lat, one, 0 * one, 0 * one, 0 * one, 4e306 * one)
     dt = float(gb.Hydro.from_lattice(lat).compute_dt(torch.from_numpy(U).cuda())[0])
     assert abs(dt / (0.8 / (2 * np.sqrt(1.4 * 4e306) / lat.dx[0])) - 1.0) <= 1e-14
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_a_flow_whose_sound_speed_is_lost(gb, sign):
+    """u + c = u: the contact speed has no value.  The cells are not finite afterwards;
+    they are not ones whose mass has stopped moving."""
+    lat = wl.lattice_2d(2, 2, 8, 8, 4, bc="periodic")
+    rng = np.random.default_rng(8)
+    rho = 2.0 ** rng.integers(0, 2, (lat.nblocks,) + lat.padded)      # so that m / rho is u
+    U = state(lat, rho, sign * 1e10 + 0 * rho, 0 * rho, 0 * rho, 1e-14 + 0 * rho)
+    h = gb.Hydro.from_lattice(lat)
+    out = torch.zeros(lat.shape, dtype=torch.float64, device="cuda")
+    h.stage(torch.from_numpy(U).cuda(), None, out, 1e-13, 0.0, 1.0)
+    zs, ys, xs = lat.interior_slices()
+    assert not torch.isfinite(out[:, 0, zs, ys, xs]).any()
