@@ -261,13 +261,15 @@ int gbh_get_prim_carry(gbh_ctx *ctx, int *enabled);
  * the coarser level).  The stage kernel then reads those fluxes
  * instead of solving each shared face in both blocks.  Results, dt and
  * floor counts are bit for bit those without it (the same face states and
- * HLLC arithmetic).  Every gbh_create* allocates its buffer ([nblocks][6]
- * [5][nxb max(nxb, nzb)] doubles) and switches it on for 3-D contexts (off
- * if that allocation fails); 2-D contexts start with it off (enable
- * allocates [nblocks][6][5][nxb] doubles).  On by default it runs where it
- * pays, for blocks narrower than 16 cells in whole-block work items; after a
- * call with enable != 0 it runs at every width.  enable = 0 switches it off (the
- * buffer stays).  GBH_ERR_NOMEM if enable != 0 and the buffer cannot be
+ * HLLC arithmetic).  Every gbh_create* switches it on for 3-D blocks narrower
+ * than 16 cells, where it pays, and allocates its buffer ([nblocks][6]
+ * [5][nxb max(nxb, nzb)] doubles; off if that allocation fails); it then runs in
+ * stages whose work items are whole blocks.  Other contexts start with it off and
+ * without the buffer (2-D: [nblocks][6][5][nxb] doubles).  After a call with
+ * enable != 0 it runs at every width, in whole-block work items.  enable = 0
+ * switches it off (the buffer stays).  gbh_get_face_prepass writes 1 to *enabled
+ * when it is on; gbh_stage_plan tells whether a stage takes it.
+ * GBH_ERR_NOMEM if enable != 0 and the buffer cannot be
  * allocated.  Drops a captured graph. */
 int gbh_set_face_prepass(gbh_ctx *ctx, int enable);
 int gbh_get_face_prepass(gbh_ctx *ctx, int *enabled);

@@ -227,6 +227,12 @@ bool take_wide(int nx, bool dim3, long long items, int sms) {
   return !dim3 || items <= 2LL * sms;
 }
 
+// Whether a stage runs the face pre-pass where the caller has not asked for it: a
+// block of 16^3 has few boundary faces for what the extra launch and its buffer
+// cost, and a block plane of 2-D fewer (us a step with it and without: 4096 blocks of
+// 16^3 11520 and 11380, 4096 of 8^3 1840 and 2040, 13824 of 4^3 1690 and 1930).
+bool prepass_pays(const Layout& L) { return L.ndim == 3 && L.nx < 16; }
+
 // What a stage launch over nblk blocks takes (0: all the blocks it would update);
 // listed: over a block list of the caller's, ranged: one of a sequence of block
 // ranges (see stage_launch).
@@ -240,12 +246,8 @@ StagePlan plan_stage(const gbh_ctx* c, int ring, bool gather, long long nblk, bo
   const Decomp d = ranged ? c->dec_range : ring == 0 || ring == 2 || ring == 4 ? c->dec[ring / 2] : Decomp{};
   if (nblk <= 0) nblk = c->refined ? c->nactive : L.nblocks;
   StagePlan p{1, 1, d.items_per_cta, d.ysplit, false, false};
-  // The face pre-pass by default only below 16 cells per side: a block of 16^3
-  // has few boundary faces for what the extra launch and its buffer cost now
-  // that a face takes 19 FP64 instructions (4096 blocks of 16^3: 12.32 ms a step
-  // with it, 12.17 without; 4096 blocks of 8^3: 1.86 and 2.09).
   p.prepass = c->face_prepass && c->d_bflux && ring == 0 && gather && (!listed || ranged) && p.ysplit == 1 &&
-              (c->prepass_asked || L.nx < 16);
+              (c->prepass_asked || prepass_pays(L));
   if (L.ndim == 3) {
     // a ring-updating stage spans nz + 2*ring planes; with the pre-pass a work item
     // is a whole block: where the caller asked for it, and in every range of a
@@ -668,16 +670,10 @@ static int step_cfl(gbh_ctx* c, double* U, double* dt_dev, cudaStream_t s, PrimC
 }
 
 
-
-// The two arrays of the primitive carry.  If they cannot
-// be allocated the carry stays off and every stage converts on load (the
-// results are the same bit for bit); returns whether it is on.
-// The face pre-pass buffer (uniform contexts); off if it cannot be allocated.
-// Switched on at creation for 3-D contexts only: in 2-D a block plane has few
-// boundary faces for what the extra launch costs (the 96-problem 2-D ensemble
-// measured 1.2% slower with it, the 256^3 3-D step 3.3% faster).
+// The face pre-pass and its buffer; off if that cannot be allocated.  Switched on
+// at creation for 3-D blocks below 16 cells per side only (prepass_pays).
 static bool alloc_face_buffer(gbh_ctx* c, bool at_create = false) {
-  if (at_create && c->lay.ndim != 3) return false;
+  if (at_create && !prepass_pays(c->lay)) return false;
   if (!c->d_bflux) {
     const size_t nf = (size_t)c->lay.nx * (c->lay.ndim == 3 ? (c->lay.nz > c->lay.nx ? c->lay.nz : c->lay.nx) : 1);
     if (cudaMalloc(&c->d_bflux, sizeof(double) * 6 * 5 * nf * (size_t)c->lay.nblocks) != cudaSuccess) {
@@ -691,6 +687,9 @@ static bool alloc_face_buffer(gbh_ctx* c, bool at_create = false) {
   return true;
 }
 
+// The two arrays of the primitive carry.  If they cannot
+// be allocated the carry stays off and every stage converts on load (the
+// results are the same bit for bit); returns whether it is on.
 static bool alloc_prim_buffers(gbh_ctx* c) {
   if (!c->d_W[0]) {
     const size_t bytes = sizeof(double) * state_elems(c->lay);

@@ -265,8 +265,9 @@ class Hydro:
         return bool(out.value)
 
     def set_face_prepass(self, enable: bool = True):
-        """Solve every block face once in a pre-pass before each interior stage
-        (on by default on 3-D uniform contexts; the results do not depend on it, bit for bit)."""
+        """Solve every block face once in a pre-pass before each interior stage (on by
+        default for 3-D blocks narrower than 16 cells, in stages of whole-block work
+        items; the results do not depend on it, bit for bit)."""
         self._check(self.lib.gbh_set_face_prepass(self.ctx, int(bool(enable))))
 
     def face_prepass(self) -> bool:
