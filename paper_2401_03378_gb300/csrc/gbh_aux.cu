@@ -22,6 +22,13 @@ __device__ __forceinline__ unsigned div_by(unsigned q, const Divisor& v) {
   return FAST ? __umulhi(q, v.m) : q / v.d;
 }
 
+// Cell (i, j, k) of a block's padded array.  In 32 bits where the divisions by
+// multiplication are exact (FAST): such a block has far fewer than 2^31 padded cells.
+template <bool FAST>
+__device__ __forceinline__ long long padded_index(const Layout& L, int i, int j, int k) {
+  return FAST ? (k * L.nyp + j) * L.nxp + i : ((long long)k * L.nyp + j) * L.nxp + i;
+}
+
 // The guard cells of a block, numbered: the z guard planes (all their cells),
 // then in every interior plane the 2 g full rows and the 2 g x guards of each
 // interior row.
@@ -106,8 +113,8 @@ __global__ void __launch_bounds__(kThreads) fill_kernel(const FillArgs a, const 
     const int si = flags & 1 ? (ox ? L.g + L.nx - 1 : L.g) : ii;
     const int sj = flags & 2 ? (oy ? L.g + L.ny - 1 : L.g) : jj;
     const int sk = flags & 4 ? (oz ? L.gz + L.nz - 1 : L.gz) : kk;
-    const long long so = GBH_IX(s_shift[e] + (sk * L.nyp + sj) * L.nxp + si, lim);
-    const long long dof = GBH_IX((long long)b * L.bstride + (kk * L.nyp + jj) * L.nxp + ii, lim);
+    const long long so = GBH_IX(s_shift[e] + padded_index<FAST>(L, si, sj, sk), lim);
+    const long long dof = GBH_IX((long long)b * L.bstride + padded_index<FAST>(L, ii, jj, kk), lim);
     if constexpr (X == 2) {
       double2 v[5];
       if (flags & 1) {
