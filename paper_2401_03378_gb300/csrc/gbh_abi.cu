@@ -230,7 +230,7 @@ bool take_wide(int nx, bool dim3, long long items, int sms) {
 // Whether a stage runs the face pre-pass where the caller has not asked for it: a
 // block of 16^3 has few boundary faces for what the extra launch and its buffer
 // cost, and a block plane of 2-D fewer (us a step with it and without: 4096 blocks of
-// 16^3 11520 and 11380, 4096 of 8^3 1840 and 2040, 13824 of 4^3 1690 and 1930).
+// 16^3 11520 and 11380, 4096 of 8^3 1840 and 2040, 13824 of 4^3 1690 and 1900).
 bool prepass_pays(const Layout& L) { return L.ndim == 3 && L.nx < 16; }
 
 // What a stage launch over nblk blocks takes (0: all the blocks it would update);

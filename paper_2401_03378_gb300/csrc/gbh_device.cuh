@@ -181,12 +181,13 @@ __device__ __forceinline__ double max_nonneg(double a, double b) {
   return bitsd((long long)(x > y ? x : y));
 }
 
-// Maximum over the NT threads of a CTA (NT a power of two) of non-negative
-// values: xor shuffles within each warp (over the lanes the CTA has), then
-// the warps' maxima through s_warp[NT/32] and one more warp of shuffles.  The
+// Maximum over the NT threads of a CTA (whole warps, at most 32, or a power of two
+// below 32) of non-negative values: xor shuffles within each warp (over the lanes the
+// CTA has), then the warps' maxima through s_warp[NT/32] and one more warp of shuffles.  The
 // result is valid in thread 0; every thread of the CTA must call it.
 template <int NT>
 __device__ __forceinline__ double block_max(double v, double* s_warp) {
+  static_assert(NT < 32 ? (NT & (NT - 1)) == 0 : NT % 32 == 0 && NT <= 1024);
   constexpr int WL = NT < 32 ? NT : 32;
   constexpr unsigned mask = WL == 32 ? 0xffffffffu : ((1u << WL) - 1u);
 #pragma unroll

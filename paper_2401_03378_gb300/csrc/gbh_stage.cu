@@ -20,7 +20,8 @@
 //    N*(N+2) y-slope cells (with the 2N faces on the block's upper x and y
 //    boundaries, which form their own face states), then the remaining N*N x
 //    faces and N*N y faces are processed as flat work lists over all threads
-//    (full warps, two passes of the CTA for the faces);
+//    (full warps, two passes of the CTA for the faces; a wide CTA has a thread per
+//    face, see stage_item);
 //  - products, quotients and roots are integer work (gbh_intmath.cuh); the FP64
 //    arithmetic left is register FMAs (gbh_fastmath.cuh);
 //  - the update of the plane reads its x/y fluxes from shared memory and its
@@ -441,8 +442,10 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
         qm[2 * os + op] = add(q3, t2, rk);
       }
     };
-    // alias: this thread's boundary flux (the list gives it one at most), kept
-    // until every read of the primitives it goes over is done
+    // alias: this thread's boundary flux (the list gives it one at most: 32 or 40 of
+    // them one after another at its end), kept until every read of the primitives it
+    // goes over is done
+    static_assert(!alias || 2 * M <= NT, "one boundary flux a thread");
     double Fb[5];
     double* ob = nullptr;
     int obv = 0;
@@ -647,9 +650,11 @@ __device__ __forceinline__ void stage_item(const StageArgs& a, int item, double*
   }
 
   if (hits) atomicAdd(a.floor_count, (unsigned long long)hits);
-  if (E == 0 && a.smax_acc) {
-    const double m = block_max<NT>(smax, s_red);   // warp shuffles, then across warps
-    if (tid == 0) atomicMax(a.smax_acc + prob, (unsigned long long)__double_as_longlong(m));
+  if constexpr (E == 0) {
+    if (a.smax_acc) {
+      const double m = block_max<NT>(smax, s_red);   // warp shuffles, then across warps
+      if (tid == 0) atomicMax(a.smax_acc + prob, (unsigned long long)__double_as_longlong(m));
+    }
   }
 }
 

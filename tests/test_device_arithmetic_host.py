@@ -6,6 +6,7 @@ import pytest
 
 from oracle import oracle as orc
 from tests.hostdevice import HostDevice
+from tests.test_hllc_arrangement import states
 
 
 @pytest.fixture(scope="module")
@@ -160,3 +161,35 @@ def test_both_sound_speeds_lost_in_the_velocities(dev, u):
 def test_receding_states_with_both_sound_speeds_lost(dev):
     L, R = np.array([1.0, -1e10, 0.0, 0.0, 1e-14]), np.array([1.0, 1e10, 0.0, 0.0, 1e-14])
     assert np.all(np.isnan(orc.hllc(L, R))) and np.all(np.isnan(dev.hllc(L, R)))
+
+
+def gas(n, seed, mach, jump):
+    rng = np.random.default_rng(seed)
+    rho, p = (10.0 ** rng.uniform(-jump, jump, n) for _ in range(2))
+    c = np.sqrt(1.4 * p / rho)
+    return np.stack([rho, *(mach * c * rng.uniform(-1, 1, n) for _ in range(3)), p], axis=1)
+
+
+@pytest.mark.parametrize("seeds,mach,tol", [((1, 2), 0.8, 1e-13), ((3, 4), 10.0, 1e-12)])
+def test_the_arrangement_of_the_kernels_against_the_textbook_flux(dev, seeds, mach, tol):
+    """Weights s / (s + rho_R) and rho_R / (s + rho_R) with s = sqrt(rho_L rho_R), the
+    Roe sound speed as a sum of non-negative terms, the star state through
+    t = S* (S_K - u_K) / (S_K - S*): the states and bounds of
+    test_hllc_arrangement.py (the textbook form's own rounding sets them)."""
+    L, R = (np.array(states(2000, k, mach)) for k in seeds)
+    got = dev.hllc(L, R)
+    for a, b, f in zip(L, R, got):
+        ref = orc.hllc(a, b)
+        assert np.max(np.abs(f - ref)) <= tol * np.max(np.abs(ref))
+
+
+def test_the_conversion_against_the_plain_formulas(dev):
+    W0 = gas(3000, 3, 10.0, 2.0)
+    rho, u, v, w, p = W0.T
+    U = np.stack([rho, rho * u, rho * v, rho * w, 2.5 * p + 0.5 * rho * (u * u + v * v + w * w)], axis=1)
+    W, hit, s = dev.prim(U)
+    assert not hit.any() and np.array_equal(W[:, 0], rho)
+    assert np.allclose(W[:, 1:4], U[:, 1:4] / rho[:, None], rtol=4e-16, atol=0)
+    assert np.all(np.abs(W[:, 4] - p) <= 1e-15 * U[:, 4])
+    ref = np.sqrt(1.4 * W[:, 4] / rho) * 6.0 + np.abs(W[:, 1]) + 2.0 * np.abs(W[:, 2]) + 3.0 * np.abs(W[:, 3])
+    assert np.allclose(s, ref, rtol=4e-15, atol=0)
