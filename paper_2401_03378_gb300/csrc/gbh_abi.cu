@@ -1640,9 +1640,11 @@ static int pipe_setup(gbh_ctx* c, bool interior) {
   // not fill the chip by themselves (the stages of neighbouring chunks run side
   // by side and fill most of it).  So about sqrt(copy time / 13 us) chunks, as a
   // power of two, with the link's 200 GB/s in each direction.  Us per step, from
-  // waves of whole blocks to this: 216 blocks of 16^3 1197 -> 1098 (4), 512: 2510 -> 2034
-  // (8), 990: 4073 -> 3681 (8), 4096: 13.0 ms (16); 1728 of 8^3 1682 -> 1417 (4); 64 of
-  // 16^3 407 -> 419 (2).
+  // waves of whole blocks to this, on one box: 216 blocks of 16^3 1197 -> 1098 (4),
+  // 512: 2510 -> 2034 (8), 990: 4073 -> 3681 (8), 4096: 13.0 ms (16); 1728 of 8^3
+  // 1682 -> 1417 (4); 64 of 16^3 407 -> 419 (2).  Boxes differ by their links: 4096
+  // blocks take 13.0 to 15.9 ms.  (With a periodic boundary in z the first range waits
+  // for the last one's copy, and 4096 blocks take 21.6.)
   int K = c->pipe_chunks_wanted;
   if (K <= 0) {
     const double copies = 2.0 * sizeof(double) * 5.0 * ((double)c->lay.nx * c->lay.ny * c->lay.nz) * NB / 200e9;

@@ -141,8 +141,9 @@ __global__ void __launch_bounds__(kThreads) fill_kernel(const FillArgs a, const 
 // atomicMax per CTA and block on the bit pattern, which orders like the
 // non-negative value).  A CTA takes one of `parts` shares of a block's cells; with
 // parts = 0 the next kThreads cells of the list's blocks one after another (blocks
-// of fewer cells; no `problem`).  nx = ny = 2^lg.  512 blocks of 16^3: 92 -> 54 us (the 64-bit divisions of a cell
-// index and 22 FP64 instructions a cell are gone).
+// of fewer cells; no `problem`).  nx = ny = 2^lg.  512 blocks of 16^3: 92 -> 55 us (the
+// 64-bit divisions of a cell index and 17 of 22 FP64 instructions a cell are gone);
+// 65536 blocks of 4^2: 39 us, 219 with a CTA to each block.
 __global__ void __launch_bounds__(kThreads) dt_reduce_kernel(const DtArgs a, const int* problem, int parts, int lg) {
   const Layout& L = a.lay;
   const unsigned per = (unsigned)(L.nx * L.ny * L.nz);

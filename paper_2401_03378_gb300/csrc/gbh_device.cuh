@@ -91,7 +91,7 @@ __device__ __forceinline__ uint32_t no_flux_mask(const double WL[5], const doubl
 // calcEos role: conserved (rho, mx, my, mz, E) -> primitive (rho, u, v, w, p),
 // p = (gamma-1) (E - (mx^2 + my^2 + mz^2) / (2 rho)).  Floors rho at small_rho and
 // p at small_p (floored_rho, floored_p) and leaves 1/rho in ir.  On the integer pipes but
-// for the subtraction: 8 FP64 instructions of 64 cycles became 1 and about 110
+// for the subtraction: 8 FP64 instructions of 64 cycles became 1 and about 200
 // more integer ones.  A conserved variable that is not finite, or beyond 2^1017, makes u,
 // v and w NaN, and p NaN or the floor (through the FP32 watch: exact tests took 0.5% of a
 // step); prim_beyond gives what the plain formulas do there.
@@ -264,9 +264,11 @@ __device__ __forceinline__ double signal_speed_ir(const double W[5], const Wide&
 // way (m_L - m_R is a sum of two negative numbers), as do m_K, h_K, rho_K t and
 // g m_K: 26 FP64 instructions a face are left (256^3 step 14.07 -> 12.33 ms).  The
 // sums of squares and the products with v_K and w_K stay on the FP64 pipe: a
-// face takes about 1050 integer instructions, and with these eight in integer
-// form too (19 FP64, 1150) the integer pipes were the longer ones inside the
-// face passes (96-problem ensemble 4.89 -> 4.73 ms, 256^3 11.74 -> 11.62 ms).
+// face takes about 960 integer instructions (gbh_op_count_probe), and with these
+// seven in integer form too (19 FP64, about 100 more) the integer pipes were the
+// longer ones inside the face passes (96-problem ensemble 4.89 -> 4.73 ms, 256^3
+// 11.74 -> 11.62 ms).  Results that can leave the range of a double go through
+// wide_signed, and no_flux_mask says where there is no flux: 0.7% of a step.
 __device__ __forceinline__ void hllc_flux(const double WL[5], const double WR[5], const Eos& e,
                                           double F[5]) {
   const Rk& k = e.k;
