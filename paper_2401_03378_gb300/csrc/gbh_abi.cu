@@ -1025,22 +1025,29 @@ int gbh_autotune(gbh_ctx* c, const double* U, int* kchunk_out, int* items_out, v
   if (c->lay.nx >= 8) splits.push_back(2);
   const long long nlist = c->refined ? c->nactive : c->lay.nblocks;
   // first what a launch chooses by itself, the default of a new context; a fixed
-  // choice has to be 2% faster, about what two timed launches can tell apart
+  // choice has to be 2% faster, about what two timed launches can tell apart, and
+  // that again beside it at the end (the first launches of an idle GPU are slow)
   auto tune = [&](int ring, const std::vector<Decomp>& fixed) {
     Decomp& d = c->dec[ring / 2];
+    const Decomp own;
     Decomp pick;
-    d = pick;
     float best = 0.f, ms = 0.f;
-    if ((rc = time_stage(c, U, ring, e0, e1, s, &best))) return;
-    best *= 0.98f;
-    for (const Decomp& t : fixed) {
+    auto timed = [&](const Decomp& t, float* out) {
       d = t;
-      if ((rc = time_stage(c, U, ring, e0, e1, s, &ms))) return;
+      return (rc = time_stage(c, U, ring, e0, e1, s, out)) == GBH_OK;
+    };
+    if (!timed(own, &best)) return;
+    best *= 0.98f;
+    bool found = false;
+    for (const Decomp& t : fixed) {
+      if (!timed(t, &ms)) return;
       if (ms < best) {
         best = ms;
         pick = t;
+        found = true;
       }
     }
+    if (found && !(timed(own, &best) && timed(pick, &ms) && ms < 0.98f * best)) pick = own;
     d = pick;
   };
   // the interior stage: z-chunk x a CTA's items x row bands, the last count of items
