@@ -190,8 +190,8 @@ def fp64_issue(inst_per_launch, ms_per_launch: float, sm_mhz, sms: int):
     lanes = inst_per_launch / (ms_per_launch / 1e3 * mhz * 1e6 * sms)
     return {"fp64_inst_per_launch": inst_per_launch, "lanes_per_sm_clock": lanes, "of_peak_lanes": lanes / 2.0,
             "sm_mhz": mhz, "sm_mhz_source": "sampled median" if sm_mhz else "nominal (no clock samples)",
-            "note": "FP64 thread instructions per zone from the ncu record of the same kernel source, "
-                    "times zones, over the CUDA-event launch time"}
+            "note": "FP64 thread instructions per zone from the ncu record of the same kernel source (at 128^3, "
+                    "whose z-chunks repeat about 3% of them), times zones, over the CUDA-event launch time"}
 
 
 def load_peaks():
